@@ -58,56 +58,55 @@ namespace {
 using namespace dev;
 using namespace tc;
 
-constexpr int NPW = 8, NCW = 8;                 // producer and consumer warps
-constexpr int NP = NPW * 32, NC = NCW * 32;
-constexpr int MMA_WARP = NPW + NCW;
-constexpr int COEF_WARP = MMA_WARP + 1;        // stages the per-visibility coefficients (float pairs)
-constexpr int NT = NP + NC + 64;
-constexpr int TV = 64;                          // visibilities per tile (rows 2 k + re/im)
-constexpr int AST = 2;                          // A stages (gated by the MMAs)
-constexpr int EST = 4;                          // Ey*, coefficient stages and accumulators (gated by the consumers)
-constexpr int T4K = 128 * 32;                   // 128 rows x 16 K FP16
-constexpr int CF_BYTES = EST * TV * 16;         // coefficients: [EST][TV] float4 (a, b, c, index)
-constexpr int PART_BYTES = 2 * 2 * 2 * 4 * TV * 4;   // consumer exchange: [2 tiles][re, im][h][4][TV] float
-static_assert(AST == 2 && EST == 4, "stage arithmetic below");
-static_assert(EST * 128 <= 512, "accumulators in tensor memory");
+constexpr int NWW = 8;                          // worker warps
+constexpr int MMA_WARP = NWW;
+constexpr int NT = NWW * 32 + 32;
+constexpr int CTAS = 2;                         // per SM
+constexpr int TV = 128;                         // visibilities per tile (rows of A and D)
+constexpr uint32_t TMEM_COLS = 256;             // two CTAs share an SM's 512
 
 // Layout for subgrid size L (32, 24 or 16)
 template <int L>
 struct SepD {
     static constexpr int SL = L, SPIX = L * L;
     static constexpr int KT = L / 8;                // K steps of 16 (8 x, re/im) over the L x
-    // B (fixed per subgrid), each [KT][4 L rows (q, y), padded to 128]: Q0 hi, Q0 lo, Q1 hi
-    static constexpr int B0H_OFF = 0, B0L_OFF = B0H_OFF + KT * T4K, B1H_OFF = B0L_OFF + KT * T4K;
-    static constexpr int A_OFF = B1H_OFF + KT * T4K;   // A: [AST][m = 0 hi, m = 0 lo, m = 1 hi][KT][128 rows]
-    static constexpr int A_STAGE = 3 * KT * T4K;
-    static constexpr int EY_OFF = A_OFF + AST * A_STAGE;   // Ey*: [2][L / 2 y pairs][TV] float4 (consumers)
-    static constexpr int EY_STAGE = L * TV * 8;
-    static constexpr int CF_OFF = EY_OFF + 2 * EY_STAGE;
-    static constexpr int PART_OFF = CF_OFF + CF_BYTES;
-    static constexpr int SMEM = PART_OFF + PART_BYTES;
-    static constexpr int FFT_P = L + 1;
-    // the subgrid's A-terms (A_p, A_q: [2][L^2] 2 x 2 complex), fetched by bulk copies at the
-    // start of the prologue beside the transform planes (A stages and Ey* table are free until
-    // the tiles)
-    static constexpr int AT_OFF = A_OFF + 4 * L * FFT_P * 8;
-    static constexpr uint32_t AT_BYTES = SPIX * 32;       // one station
-    static constexpr uint32_t IDESC_N = idesc_m128(4 * L);
-    // B tasks of the prologue: (q, y block of 8, x chunk of 4), one core matrix each
-    static constexpr int YB = L / 8, XC = L / 4, NTASK = 4 * YB * XC;
-    static constexpr int NWT = (NTASK + MMA_WARP - 1) / MMA_WARP;
-    static constexpr int EYP = L * TV / NC / 2;     // Ey* pairs per consumer thread
+    // a tile's products go in PARTS rounds of QH polarisations into one accumulator of PN columns
+    static constexpr int QH = L == 16 ? 4 : 2, PARTS = 4 / QH, PN = QH * 2 * L;
+    // D column (B row) of (q', y, re/im) in a part: 2 L q' + 2 YB (y / YB) + YB (re/im) + y % YB
+    static constexpr int YB = L == 24 ? 4 : 8;
+    // B (fixed per subgrid), each [KT][part][PN rows][16 K]: Q0 hi, Q0 lo, Q1 hi
+    static constexpr int TB = 8 * L * 32;           // one K step: 8 L rows x 32 bytes
+    static constexpr int B0L = KT * TB, B1H = 2 * KT * TB, B_BYTES = 3 * KT * TB;
+    // prologue scratch over B: the subgrid's grid rows, then the transform planes
+    static constexpr int FFT_P = L + 1, FFT_OFF = SPIX * 32, FFT_BYTES = 4 * L * FFT_P * 8;
+    static constexpr int PART_OFF = B_BYTES > FFT_OFF + FFT_BYTES ? B_BYTES : FFT_OFF + FFT_BYTES;
+    static constexpr int SEP_OFF = PART_OFF + 2 * 2 * TV * 16;   // [2 tiles][2 pol pairs][TV] float4 (y halves meet)
+    static constexpr int SMEM = SEP_OFF + 2 * (L / 2) * 16;      // (X, X + 1, s(X), s(X + 1)) per x pair, t alike
+    // tensor memory: accumulator, then A hi, lo and m = 1, one column per x
+    static constexpr uint32_t A_COL = PN;
+    static constexpr uint32_t IDESC = idesc_m128(PN);
+    // a worker's half of the x (A) and of the y (sum) of its visibility, in chunks
+    static constexpr int H = L / 2, XCH = H % 8 == 0 ? 8 : 4;
+    // image pixels by worker warp: tiles of 8 y x 4 x, one B core matrix row set per warp store
+    static constexpr int NTILE = (L / 8) * (L / 4), TPW = (NTILE + NWW - 1) / NWW;
     static_assert(L == 32 || L == 24 || L == 16, "subgrid sizes of the separable kernels");
-    static_assert(4 * L * FFT_P * 8 <= AST * A_STAGE, "transform planes fit over the A stages");
-    static_assert(AT_OFF % 16 == 0 && AT_OFF + 2 * (int)AT_BYTES <= CF_OFF, "A-terms before the coefficient stages");
-    static_assert(3 * KT * T4K >= SPIX * 32, "the subgrid's grid rows fit in the B area");
+    static_assert(A_COL + 3 * L <= TMEM_COLS, "accumulator and A in the CTA's tensor memory");
+    static_assert(PN % 16 == 0 && PN <= 256, "MMA N");
+    static_assert(H % YB == 0 && H % XCH == 0, "whole chunks per worker");
+    static_assert(FFT_OFF % 16 == 0 && PART_OFF % 16 == 0, "16-byte aligned areas");
+    static_assert(CTAS * (SMEM + 2048) <= 227 * 1024, "shared memory of the SM's CTAs");
     static_assert(L <= 32, "one grid row per lane of warp 0");
-    static_assert(4 * L <= 128 && (4 * L) % 16 == 0, "B rows (q, y) in one MMA");
-    static_assert(L * TV % (2 * NC) == 0 && (L / 2) % 4 == 0, "Ey* pairs spread evenly over the consumers");
-    static_assert(L % 8 == 0 && 4 * NPW >= L, "x columns over the producer warps");
 };
 
-__device__ __forceinline__ void consumers_sync() { asm volatile("bar.sync 2, %0;" :: "n"(NC) : "memory"); }
+// the two warps of a lane quarter (constant barrier numbers: a register would reserve all 16)
+__device__ __forceinline__ void pair_sync(int quarter) {
+    switch (quarter) {
+    case 0: asm volatile("bar.sync 1, 64;" ::: "memory"); break;
+    case 1: asm volatile("bar.sync 2, 64;" ::: "memory"); break;
+    case 2: asm volatile("bar.sync 3, 64;" ::: "memory"); break;
+    default: asm volatile("bar.sync 4, 64;" ::: "memory"); break;
+    }
+}
 
 // Visibilities of subgrid d of geometry g from its image src[L][L][4], or with
 // FUSED from the grid src[layer][N][N][4]: split and transformed in shared memory
@@ -118,119 +117,84 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
                                                    const float4 *__restrict__ aterms, const float *__restrict__ taper,
                                                    float4 *__restrict__ vis_out) {
     using C = SepD<L>;
-    constexpr int SL = C::SL, SPIX = C::SPIX, KT = C::KT, B0H_OFF = C::B0H_OFF, B0L_OFF = C::B0L_OFF;
-    constexpr int B1H_OFF = C::B1H_OFF, A_OFF = C::A_OFF, A_STAGE = C::A_STAGE, EY_OFF = C::EY_OFF;
-    constexpr int CF_OFF = C::CF_OFF, PART_OFF = C::PART_OFF, FFT_P = C::FFT_P, AT_OFF = C::AT_OFF;
-    constexpr uint32_t AT_BYTES = C::AT_BYTES;
+    constexpr int SL = C::SL, SPIX = C::SPIX, KT = C::KT, FFT_P = C::FFT_P, H = C::H, YB = C::YB, QH = C::QH;
     extern __shared__ __align__(1024) uint8_t smem[];
-    float2 *s_fft = (float2 *)(smem + A_OFF);       // [4][L][L + 1] during the prologue
-    float4 *s_coef = (float4 *)(smem + CF_OFF);
-    float4 *s_ey = (float4 *)(smem + EY_OFF);
-    float *s_part = (float *)(smem + PART_OFF);
+    float2 *s_fft = (float2 *)(smem + C::FFT_OFF);       // [4][L][L + 1] during the prologue
+    float4 *s_part = (float4 *)(smem + C::PART_OFF);
+    float4 *s_sep = (float4 *)(smem + C::SEP_OFF);       // x pairs, then y pairs
     __shared__ uint32_t s_tmem;
-    __shared__ __align__(8) uint64_t s_afull[AST], s_aempty[AST], s_eyfull[EST], s_eyempty[EST], s_dfull[EST],
-        s_dempty[EST], s_drain, s_atbar, s_gbar;
-    __shared__ float s_red[NT / 32];
+    __shared__ __align__(8) uint64_t s_afull, s_dfull, s_dempty, s_drain, s_gbar;
+    __shared__ float s_red[NWW];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int n_tiles = (d.kp + TV - 1) / TV;
+    const int kp = d.kp, n_tiles = (kp + TV - 1) / TV;
 
     if (warp == MMA_WARP) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     :: "r"(smem_u32(&s_tmem)), "n"(512));
+                     :: "r"(smem_u32(&s_tmem)), "n"(TMEM_COLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (warp == 0) {
-        // barriers by lane 0; the copies are then issued by the whole warp, one per lane: the
-        // subgrid's 32 grid rows (1 KB each, contiguous in the grid) into the B area, which is
-        // free until B is formed at the end of the prologue, and the two stations' A-terms
+        // barriers by lane 0; then one bulk copy per lane: the subgrid's grid rows (32 L bytes
+        // each, contiguous in the grid)
         if (lane == 0) {
-            for (int s = 0; s < AST; ++s) {
-                mbar_init(smem_u32(&s_afull[s]), NPW);
-                mbar_init(smem_u32(&s_aempty[s]), 1);
-            }
-            for (int e = 0; e < EST; ++e) {
-                mbar_init(smem_u32(&s_eyfull[e]), 1);
-                mbar_init(smem_u32(&s_eyempty[e]), NCW);
-                mbar_init(smem_u32(&s_dfull[e]), 1);
-                mbar_init(smem_u32(&s_dempty[e]), NCW);
-            }
+            mbar_init(smem_u32(&s_afull), NWW);
+            mbar_init(smem_u32(&s_dfull), 1);
+            mbar_init(smem_u32(&s_dempty), NWW);
             mbar_init(smem_u32(&s_drain), 1);
-            mbar_init(smem_u32(&s_atbar), 1);
             mbar_init(smem_u32(&s_gbar), 1);
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-            if (FUSED) mbar_expect_tx(smem_u32(&s_gbar), SL * SL * 32);
-            if (aterms) mbar_expect_tx(smem_u32(&s_atbar), 2 * AT_BYTES);
+            if (FUSED) mbar_expect_tx(smem_u32(&s_gbar), SPIX * 32);
         }
         __syncwarp();
         if (FUSED && lane < SL) {
             const float4 *gsrc = src + (size_t)d.layer * g.N * g.N * 2;
-            bulk_g2s(smem_u32(smem + B0H_OFF + lane * SL * 32), gsrc + 2 * ((size_t)(d.r0 + lane) * g.N + d.q0),
-                     SL * 32, smem_u32(&s_gbar));
-        }
-        if (aterms && lane < 2) {
-            const float4 *base = aterms + 2 * ((size_t)d.slot * g.n_stations) * SPIX;
-            bulk_g2s(smem_u32(smem + AT_OFF + lane * AT_BYTES), base + 2 * (size_t)(lane ? d.st_q : d.st_p) * SPIX,
-                     AT_BYTES, smem_u32(&s_atbar));
+            bulk_g2s(smem_u32(smem + lane * SL * 32), gsrc + 2 * ((size_t)(d.r0 + lane) * g.N + d.q0), SL * 32,
+                     smem_u32(&s_gbar));
         }
     }
+    if (tid < SL) {
+        const float X = (float)((2 * tid) % SL - SL / 2);
+        s_sep[tid] = make_float4(X, X + 1.0f, g.sep[2 * tid], g.sep[2 * tid + 1]);
+    }
 
-    // the coefficient warp loads its first tile's coordinates now, so that they have
-    // arrived when the tiles start
-    struct Raw {
-        float4 uv, sc;
-        float2 w;
-        uint32_t vi;
-        bool in, flag;
-    };
+    // workers: visibility 32 (warp % 4) + lane of the tile, x and y half warp / 4
+    const int quarter = warp & 3, half = warp >> 2, row = 32 * quarter + lane;
+    // its coordinates, loaded one tile ahead (the first tile's before the prologue)
     const float4 *uvw2 = (const float4 *)g.uvw_f2;
     const float4 *sc2 = (const float4 *)g.scale_f2;
-    auto load_raw = [&](Raw &r, int k) {
-        r.in = k < d.kp;
-        r.flag = false;
-        if (r.in) {
-            int tt, c;
-            const size_t vi = vis_index(g, d, k, tt, c);
-            const size_t bt = (size_t)d.bl * g.n_t + tt;
-            r.uv = uvw2[2 * bt];
-            const float4 w4 = uvw2[2 * bt + 1];
-            r.w = make_float2(w4.x, w4.y);
-            r.sc = sc2[c];
-            r.vi = (uint32_t)vi;
-            r.flag = flags && flags[vi];
+    const int dt = TV / d.nc, dc = TV - dt * d.nc;
+    int vt = row / d.nc, vc = row - vt * d.nc;           // timestep and channel in the subgrid
+    float4 ruv = make_float4(0.f, 0.f, 0.f, 0.f), rsc = ruv;
+    float2 rw = make_float2(0.f, 0.f);
+    uint32_t rvi = 0xFFFFFFFFu;                          // output index, bit 31 = flagged; all ones: none
+    auto load_raw = [&](int k) {
+        rvi = 0xFFFFFFFFu;
+        if (k < kp) {
+            const size_t bt = (size_t)d.bl * g.n_t + d.t0 + vt;
+            const int c = d.c0 + vc;
+            ruv = uvw2[2 * bt];
+            rw = *(const float2 *)(uvw2 + 2 * bt + 1);
+            rsc = sc2[c];
+            rvi = (uint32_t)(bt * g.n_chan + c);
+            if (flags && flags[rvi]) rvi |= 0x80000000u;
+        }
+        vt += dt;
+        vc += dc;
+        if (vc >= d.nc) {
+            vc -= d.nc;
+            ++vt;
         }
     };
-    Raw r0 = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f), make_float2(0.f, 0.f), 0u, false,
-              false},
-        r1 = r0;
-    if (warp == COEF_WARP && n_tiles > 0) {
-        load_raw(r0, lane);
-        load_raw(r1, lane + 32);
-    }
-    // the prologue's other global reads, issued while the copies run: the taper of this
-    // thread's pixels and the remainder r(x, y) of its B entries
-    constexpr int NPIX = (SPIX + NT - 1) / NT;
-    float tw_pre[NPIX];
-#pragma unroll
-    for (int i = 0; i < NPIX; ++i) tw_pre[i] = tid + i * NT < SPIX ? taper[tid + i * NT] : 0.0f;
-    constexpr int NWT = C::NWT;
-    float rr_pre[NWT];
-#pragma unroll
-    for (int i = 0; i < NWT; ++i) {
-        const int wt = warp + MMA_WARP * i;
-        const int yb = (wt / C::XC) % C::YB, xc = wt % C::XC;
-        rr_pre[i] = warp < MMA_WARP && wt < C::NTASK
-                        ? g.sep[2 * SL + (8 * yb + (lane >> 2)) * SL + 4 * xc + (lane & 3)]
-                        : 0.0f;
-    }
-    __syncthreads();      // the copies' barriers are initialised
+    if (warp < NWW) load_raw(row);
+    __syncthreads();      // the copies' barrier is initialised
 
-    // ---- prologue: the corrected image P = taper A_p I A_q^H into the planes
+    // ---- prologue: the corrected image P = taper A_p I A_q^H, this thread's pixels in registers
     if (FUSED) {
         bool late = false;
         wait_or_fail(smem_u32(&s_gbar), 0u, late);
         if (late) atomicExch(&g_sepd_error, 1);
-        const float4 *rows = (const float4 *)(smem + B0H_OFF);
+        const float4 *rows = (const float4 *)smem;
         for (int pix = tid; pix < SPIX; pix += NT) {
             const int i = pix / SL, j = pix % SL;
             const float sg = ((i + j) & 1) ? -1.0f : 1.0f;
@@ -246,302 +210,280 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
         else
             fft2_planar<SL, +1>(s_fft, tid, NT);
     }
-    if (aterms) {
-        bool late = false;
-        wait_or_fail(smem_u32(&s_atbar), 0u, late);
-        if (late) atomicExch(&g_sepd_error, 1);
-    }
-    float m = 0.0f;
+    M22 P[C::TPW];
+    if (warp < NWW) {
+        float m = 0.0f;
 #pragma unroll
-    for (int ip = 0; ip < NPIX; ++ip) {
-        const int pix = tid + ip * NT;
-        if (pix >= SPIX) break;
-        const int y = pix / SL, x = pix % SL;
-        M22 P;
-        if (FUSED) {      // (-1)^(x+y) / L^2 of the transform
-            const float sg = ((x + y) & 1) ? -1.0f / SPIX : 1.0f / SPIX;
+        for (int i = 0; i < C::TPW; ++i) {
+            const int tile = warp + NWW * i;
+            if (tile >= C::NTILE) break;
+            const int y = 8 * (tile / (SL / 4)) + (lane >> 2), x = 4 * (tile % (SL / 4)) + (lane & 3), pix = y * SL + x;
+            if (FUSED) {      // (-1)^(x+y) / L^2 of the transform
+                const float sg = ((x + y) & 1) ? -1.0f / SPIX : 1.0f / SPIX;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float2 v = s_fft[(q * SL + y) * FFT_P + x];
+                    P[i].m[q] = make_float2(sg * v.x, sg * v.y);
+                }
+            } else {
+                P[i] = load_m22(src + 2 * pix);
+            }
+            if (d.dws != 0.0f) {      // the sums use w_s: the rest of the w offset, exp(-i 2 pi (w_s - w0) n')
+                float sn, cs;
+                sincospif(d.dws * g.nprime[pix], &sn, &cs);     // (dws in half turns: exact reduction)
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    P[i].m[q] = make_float2(P[i].m[q].x * cs + P[i].m[q].y * sn, P[i].m[q].y * cs - P[i].m[q].x * sn);
+            }
+            if (aterms) {
+                const float4 *base = aterms + 2 * ((size_t)d.slot * g.n_stations) * SPIX + 2 * pix;
+                const M22 Ap = load_m22(base + 2 * (size_t)d.st_p * SPIX);
+                const M22 Aq = load_m22(base + 2 * (size_t)d.st_q * SPIX);
+                P[i] = mul_mul_herm(Ap, P[i], Aq);
+            }
+            const float tw = taper[pix];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const float2 v = s_fft[(q * SL + y) * FFT_P + x];
-                P.m[q] = make_float2(sg * v.x, sg * v.y);
+                P[i].m[q] = make_float2(tw * P[i].m[q].x, tw * P[i].m[q].y);
+                m = fmaxf(m, fmaxf(fabsf(P[i].m[q].x), fabsf(P[i].m[q].y)));
             }
-        } else {
-            P = load_m22(src + 2 * pix);
         }
-        if (d.dws != 0.0f) {      // the sums use w_s: the rest of the w offset, exp(-i 2 pi (w_s - w0) n')
-            float sn, cs;
-            sincospif(d.dws * g.nprime[pix], &sn, &cs);     // (dws in half turns: exact reduction)
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-                P.m[q] = make_float2(P.m[q].x * cs + P.m[q].y * sn, P.m[q].y * cs - P.m[q].x * sn);
-        }
-        if (aterms) {
-            const float4 *at = (const float4 *)(smem + AT_OFF);
-            const M22 Ap = load_m22(at + 2 * pix);
-            const M22 Aq = load_m22(at + 2 * (SPIX + pix));
-            P = mul_mul_herm(Ap, P, Aq);
-        }
-        const float tw = tw_pre[ip];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float2 v = make_float2(tw * P.m[q].x, tw * P.m[q].y);
-            s_fft[(q * SL + y) * FFT_P + x] = v;
-            m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
-        }
+        for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+        if (lane == 0) s_red[warp] = m;
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-    if (lane == 0) s_red[warp] = m;
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
+    __syncthreads();      // every pixel is in registers: the scratch area may become B
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = s_tmem;
-    m = 0.0f;
+    float inv_scale;
+    {
+        float m = 0.0f;
 #pragma unroll
-    for (int w = 0; w < NT / 32; ++w) m = fmaxf(m, s_red[w]);
-    int e2 = 0;
-    if (m > 0.0f) frexpf(m, &e2);
-    const float scale = ldexpf(1.0f, 10 - e2);
-    const float inv_scale = ldexpf(1.0f, e2 - 10);
-    // B: Q0 = scale P (hi and lo), Q1 = scale r P / sigma (hi), rows L q + y; one core matrix
-    // (8 rows y, 4 x) per warp store: warp-task wt = (q, y block, x chunk of 4)
-    if (warp < MMA_WARP) {
-        const float rs = scale / g.c_scale;
+        for (int w = 0; w < NWW; ++w) m = fmaxf(m, s_red[w]);
+        int e2 = 0;
+        if (m > 0.0f) frexpf(m, &e2);
+        const float scale = ldexpf(1.0f, 10 - e2);
+        inv_scale = ldexpf(1.0f, e2 - 10);
+        // B: Q0 = scale P (hi and lo), Q1 = scale r P / sigma (hi).  Row re of (q, y) is (Re Q, Im Q)
+        // over K = (x, cs/sn), row im (Im Q, -Re Q): the re row's halves swapped, the new high one negated
+        if (warp < NWW) {
+            const float rs = scale / g.c_scale;
 #pragma unroll
-        for (int i = 0; i < NWT; ++i) {
-            const int wt = warp + MMA_WARP * i;
-            if (wt >= C::NTASK) break;
-            const int q = wt / (C::YB * C::XC), yb = (wt / C::XC) % C::YB, xc = wt % C::XC;
-            const int y = 8 * yb + (lane >> 2), x = 4 * xc + (lane & 3);
-            const float2 p = s_fft[(q * SL + y) * FFT_P + x];
-            const float rr = rr_pre[i] * rs;
-            uint32_t h0, l0;
-            split_e(p.x * scale, p.y * scale, h0, l0);
-            const uint32_t h1 = pack_f16x2(p.x * rr, p.y * rr);
-            const uint32_t off = (uint32_t)(C::YB * q + yb) * kSBO + (uint32_t)(xc & 1) * kLBO + (uint32_t)(lane >> 2) * 16 +
-                                 (uint32_t)(lane & 3) * 4;
-            const int kk = xc >> 1;
-            *(uint32_t *)(smem + B0H_OFF + kk * T4K + off) = h0;
-            *(uint32_t *)(smem + B0L_OFF + kk * T4K + off) = l0;
-            *(uint32_t *)(smem + B1H_OFF + kk * T4K + off) = h1;
+            for (int i = 0; i < C::TPW; ++i) {
+                const int tile = warp + NWW * i;
+                if (tile >= C::NTILE) break;
+                const int y = 8 * (tile / (SL / 4)) + (lane >> 2), x = 4 * (tile % (SL / 4)) + (lane & 3);
+                const float rr = g.sep[2 * SL + y * SL + x] * rs;
+                uint8_t *Bx = smem + (x >> 3) * C::TB + ((x >> 2) & 1) * kLBO + (x & 3) * 4;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float2 p = P[i].m[q];
+                    uint32_t h0, l0;
+                    split_e(p.x * scale, p.y * scale, h0, l0);
+                    const uint32_t h1 = pack_f16x2(p.x * rr, p.y * rr);
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        const int n = 2 * SL * q + 2 * YB * (y / YB) + YB * r + y % YB;
+                        uint8_t *b = Bx + (n >> 3) * kSBO + (n & 7) * 16;
+                        *(uint32_t *)b = r ? __byte_perm(h0, 0u, 0x1032u) ^ 0x80000000u : h0;
+                        *(uint32_t *)(b + C::B0L) = r ? __byte_perm(l0, 0u, 0x1032u) ^ 0x80000000u : l0;
+                        *(uint32_t *)(b + C::B1H) = r ? __byte_perm(h1, 0u, 0x1032u) ^ 0x80000000u : h1;
+                    }
+                }
+            }
         }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();      // B complete; the planes (over the A stages) are free
+    __syncthreads();      // B complete
 
     bool failed = false;
     if (warp == MMA_WARP) {
         if (lane == 0) {
-            const uint64_t da0 = smem_desc(smem_u32(smem + A_OFF));
-            const uint64_t db0 = smem_desc(smem_u32(smem + B0H_OFF));
+            const uint64_t db0 = smem_desc(smem_u32(smem));
+            const uint32_t at = tmem + C::A_COL;
             for (int t = 0; t < n_tiles; ++t) {
-                const int s = t & 1, e = t & 3;
-                wait_or_fail(smem_u32(&s_afull[s]), (uint32_t)((t >> 1) & 1), failed);
-                if (t >= EST) wait_or_fail(smem_u32(&s_dempty[e]), (uint32_t)(((t >> 2) - 1) & 1), failed);
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t dt = tmem + 128u * (uint32_t)e;
+                wait_or_fail(smem_u32(&s_afull), (uint32_t)(t & 1), failed);
+                for (int p = 0; p < C::PARTS; ++p) {
+                    const int n = t * C::PARTS + p;
+                    if (n > 0) wait_or_fail(smem_u32(&s_dempty), (uint32_t)((n - 1) & 1), failed);
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint64_t dbp = db0 + (uint64_t)((p * C::PN * 32) >> 4);
 #pragma unroll
-                for (int kk = 0; kk < KT; ++kk) {
-                    const uint64_t da = da0 + (uint64_t)((s * A_STAGE + kk * T4K) >> 4);     // m = 0 hi
-                    const uint64_t db = db0 + (uint64_t)((kk * T4K) >> 4);                  // Q0 hi
-                    mma_ss_i(dt, da, db, C::IDESC_N, kk > 0 ? 1u : 0u);
-                    mma_ss_i(dt, da, db + (uint64_t)((KT * T4K) >> 4), C::IDESC_N, 1u);        // Q0 lo
-                    mma_ss_i(dt, da + (uint64_t)((KT * T4K) >> 4), db, C::IDESC_N, 1u);        // m = 0 lo
-                    mma_ss_i(dt, da + (uint64_t)((2 * KT * T4K) >> 4), db + (uint64_t)((2 * KT * T4K) >> 4),
-                             C::IDESC_N, 1u);                                                // m = 1 hi x Q1 hi
+                    for (int kk = 0; kk < KT; ++kk) {
+                        const uint64_t db = dbp + (uint64_t)((kk * C::TB) >> 4);
+                        const uint32_t ak = at + 8u * kk;
+                        mma_ta_i(tmem, ak, db, C::IDESC, kk > 0 ? 1u : 0u);                                 // hi x Q0 hi
+                        mma_ta_i(tmem, ak, db + (uint64_t)(C::B0L >> 4), C::IDESC, 1u);                     // hi x Q0 lo
+                        mma_ta_i(tmem, ak + SL, db, C::IDESC, 1u);                                          // lo x Q0 hi
+                        mma_ta_i(tmem, ak + 2 * SL, db + (uint64_t)(C::B1H >> 4), C::IDESC, 1u);            // m = 1
+                    }
+                    commit(smem_u32(&s_dfull));
                 }
-                commit(smem_u32(&s_aempty[s]));
-                commit(smem_u32(&s_dfull[e]));
             }
             commit(smem_u32(&s_drain));
             bool drained = false;
             wait_or_fail(smem_u32(&s_drain), 0u, drained);     // bounded: let own MMAs finish before the free
         }
         failed = __shfl_sync(0xffffffffu, failed, 0);
-    } else if (warp < NPW) {
-        // ---- producers: coefficients, A (2 x 2 embedding of Ex*) and the Ey* table per tile.
-        // A rows are (re/im, k): row k = (Re E, -Im E), row 64 + k = (Im E, Re E).  Lane = 4 k_lo + x_lo:
-        // warp w owns x = 4 w + x_lo (K step w / 2, chunk w % 2) and writes visibilities 8 kg + k_lo
-        const int klo = lane >> 2, xlo = lane & 3, x = 4 * warp + xlo;
-        const bool x_ok = SL == 32 || 4 * warp < SL;    // warps past the last x only keep the protocol
-        const float Xv = (float)(x - SL / 2), sx = g.sep[x_ok ? x : 0], csig = g.c_scale;
-        const uint32_t a_off = (uint32_t)(warp >> 1) * T4K + (uint32_t)(warp & 1) * kLBO + (uint32_t)klo * 16 +
-                               (uint32_t)xlo * 4;
-        for (int t = 0; t < n_tiles; ++t) {
-            const int s = t & 1, e = t & 3;
-            if (t >= AST) wait_or_fail(smem_u32(&s_aempty[s]), (uint32_t)(((t >> 1) - 1) & 1), failed);
-            wait_or_fail(smem_u32(&s_eyfull[e]), (uint32_t)((t >> 2) & 1), failed);      // the tile's coefficients
-            const float4 *cf = s_coef + e * TV;
-            uint8_t *As = smem + A_OFF + s * A_STAGE;
-#pragma unroll 2
-            for (int kg = 0; kg < TV / 8; ++kg) {
-                if (!x_ok) break;
-                const float4 c = cf[8 * kg + klo];
-                float sn, cs;
-                __sincosf(fmaf(c.z, sx, c.x * Xv), &sn, &cs);
-                // m = 0: a = E = cs - i sn: row re = (cs, sn), row im = (-sn, cs); the im row is the re
-                // row with halves swapped and the new low half negated (exact for FP16 parts)
-                uint32_t hr, lr;
-                split_e(cs, sn, hr, lr);
-                const uint32_t hm = __byte_perm(hr, 0u, 0x1032u) ^ 0x8000u;
-                const uint32_t lm = __byte_perm(lr, 0u, 0x1032u) ^ 0x8000u;
-                // m = 1: a = -i c sigma E = -c sigma (sn + i cs): row re = (-c sigma sn, c sigma cs)
-                const float cz = c.z * csig;
-                const uint32_t h1r = pack_f16x2(-cz * sn, cz * cs);
-                const uint32_t h1m = __byte_perm(h1r, 0u, 0x1032u) ^ 0x8000u;
-                const uint32_t o_re = a_off + (uint32_t)kg * kSBO, o_im = o_re + 8 * kSBO;
-                *(uint32_t *)(As + o_re) = hr;
-                *(uint32_t *)(As + o_im) = hm;
-                *(uint32_t *)(As + KT * T4K + o_re) = lr;
-                *(uint32_t *)(As + KT * T4K + o_im) = lm;
-                *(uint32_t *)(As + 2 * KT * T4K + o_re) = h1r;
-                *(uint32_t *)(As + 2 * KT * T4K + o_im) = h1m;
-            }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&s_afull[s]));
-        }
-        if (failed && lane == 0) atomicExch(&g_sepd_error, 1);
-    } else if (warp == COEF_WARP) {
-        // ---- coefficients: lane l stages visibilities l and l + 32 of each tile: (a, b, c) from
-        // float pairs (error-free FP32 products and sums, rounded once) and the output index (flag
-        // in bit 31); the coordinates of the next tile are loaded while this one is formed, and a
-        // stage is reused once the consumers release it (the first tile's were loaded before
-        // the prologue)
-        auto form = [&](const Raw &r) {
-            float4 cf = make_float4(0.f, 0.f, 0.f, __uint_as_float(0xFFFFFFFFu));   // beyond K_p: no output
-            if (r.in) {
-                cf.x = pair_coef(r.uv.x, r.uv.y, r.sc.x, r.sc.y, d.a0h, d.a0l);
-                cf.y = pair_coef(r.uv.z, r.uv.w, r.sc.x, r.sc.y, d.b0h, d.b0l);
-                cf.z = pair_coef(r.w.x, r.w.y, r.sc.z, r.sc.w, d.csh, d.csl);
-                cf.w = __uint_as_float(r.vi | (r.flag ? 0x80000000u : 0u));
-            }
-            return cf;
-        };
-        for (int t = 0; t < n_tiles; ++t) {
-            const int e = t & 3;
-            const float4 c0 = form(r0), c1 = form(r1);
-            if (t + 1 < n_tiles) {
-                load_raw(r0, (t + 1) * TV + lane);
-                load_raw(r1, (t + 1) * TV + lane + 32);
-            }
-            if (t >= EST) wait_or_fail(smem_u32(&s_eyempty[e]), (uint32_t)(((t >> 2) - 1) & 1), failed);
-            s_coef[e * TV + lane] = c0;
-            s_coef[e * TV + lane + 32] = c1;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&s_eyfull[e]));
-        }
-        if (failed && lane == 0) atomicExch(&g_sepd_error, 1);
     } else {
-        // ---- consumers: row 32 (warp % 4) + lane = (re/im = row / 64, k = row % 64) of the tile,
-        // polarisations 2 h, 2 h + 1; the re and im rows of a visibility meet through s_part
-        const int qq = warp & 3, h = (warp - NPW) >> 2;
-        const int ci = qq >> 1, kl = 32 * (qq & 1) + lane;
-        const uint32_t lane_base = tmem + ((uint32_t)(32 * qq) << 16);
-        // Ey* entries: visibility ke = ctid % TV, rows y = 2 p, 2 p + 1 of the pairs p = ctid / TV + 4 j
-        // (ctid = consumer thread index); entry (p, k) = (cs_2p, cs_2p+1, -sn_2p, -sn_2p+1)
-        const int ctid = tid - NP, ke = ctid & (TV - 1), p0 = ctid >> 6;
-        constexpr int EYP = C::EYP;               // pairs per thread
-        float tys[2 * EYP];
-#pragma unroll
-        for (int j = 0; j < EYP; ++j) {
-            tys[2 * j] = g.sep[SL + 2 * (p0 + 4 * j)];
-            tys[2 * j + 1] = g.sep[SL + 2 * (p0 + 4 * j) + 1];
-        }
+        const uint32_t lane_base = tmem + ((uint32_t)(32 * quarter) << 16);
+        const float csig = g.c_scale;
+        const float4 *xs = s_sep + half * (H / 2), *yt = s_sep + (SL + half * H) / 2;
+        // phase coefficients of the tile's visibility from float pairs (error-free products and
+        // sums, rounded once), and its output index; formed one tile ahead, while MMAs run
+        float ca = 0.f, cb = 0.f, cc = 0.f;
+        uint32_t vi = 0xFFFFFFFFu;
+        auto form_coef = [&](float &a, float &b, float &c, uint32_t &v) {
+            a = b = c = 0.f;
+            v = rvi;
+            if (rvi != 0xFFFFFFFFu) {
+                a = pair_coef(ruv.x, ruv.y, rsc.x, rsc.y, d.a0h, d.a0l);
+                b = pair_coef(ruv.z, ruv.w, rsc.x, rsc.y, d.b0h, d.b0l);
+                c = pair_coef(rw.x, rw.y, rsc.z, rsc.w, d.csh, d.csl);
+            }
+        };
+        // the two y halves of a visibility meet: each half's warp finishes two polarisations, own
+        // their sums over its y, the other half's through shared memory (after the next tile's A)
+        float4 own = make_float4(0.f, 0.f, 0.f, 0.f);
+        uint32_t ovi = 0xFFFFFFFFu;
+        auto finish = [&](int t) {
+            pair_sync(quarter);
+            const float4 o = s_part[((t & 1) * 2 + half) * TV + row];
+            if (ovi != 0xFFFFFFFFu && !failed) {
+                float4 v = make_float4((own.x + o.x) * inv_scale, (own.y + o.y) * inv_scale, (own.z + o.z) * inv_scale,
+                                       (own.w + o.w) * inv_scale);
+                if (ovi & 0x80000000u) v = make_float4(0.f, 0.f, 0.f, 0.f);      // flagged
+                vis_out[2 * (size_t)(ovi & 0x7FFFFFFFu) + half] = v;
+            }
+        };
+        form_coef(ca, cb, cc, vi);
+        load_raw(TV + row);
         for (int t = 0; t < n_tiles; ++t) {
-            const int s = t & 1, e = t & 3;
-            wait_or_fail(smem_u32(&s_eyfull[e]), (uint32_t)((t >> 2) & 1), failed);
-            // Ey*_k(y) = exp(-i (b_k Y + c_k t(y))) of the tile (entry y TV + k), while its MMAs run
-            float4 *eyw = s_ey + s * (SL / 2 * TV);     // [L / 2 pairs][TV]
-            {
-                const float4 c = s_coef[e * TV + ke];
-#pragma unroll
-                for (int j = 0; j < EYP; ++j) {
-                    const int pp = p0 + 4 * j;
-                    float sn0, cs0, sn1, cs1;
-                    __sincosf(fmaf(c.z, tys[2 * j], c.y * (float)(2 * pp - SL / 2)), &sn0, &cs0);
-                    __sincosf(fmaf(c.z, tys[2 * j + 1], c.y * (float)(2 * pp + 1 - SL / 2)), &sn1, &cs1);
-                    eyw[pp * TV + ke] = make_float4(cs0, cs1, -sn0, -sn1);
-                }
-            }
-            consumers_sync();
-            wait_or_fail(smem_u32(&s_dfull[e]), (uint32_t)((t >> 2) & 1), failed);
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const ulonglong2 *ey = (const ulonglong2 *)eyw;
-            // [q'][(sum er T, sum ei T)], each as packed partial sums over the even and odd rows y
-            f2_t accp[2][2];
-#pragma unroll
-            for (int q2 = 0; q2 < 2; ++q2) accp[q2][0] = accp[q2][1] = 0ull;
+            const bool active = t * TV + 32 * quarter < kp;      // the same for the whole warp
+            // A: this half's x of the visibility's row (the last part of the previous tile was waited
+            // for below, so the MMAs are done with A)
+            if (active) {
+                const float cz = cc * csig;
+                const f2_t ca2 = f2_pack(ca, ca), cc2 = f2_pack(cc, cc), cz2 = f2_pack(-cz, cz);
+                constexpr int XCH = C::XCH;
 #pragma unroll 1
-            for (int yc = 0; yc < SL / 8; ++yc) {    // rows y in [8 yc, 8 yc + 8)
-                uint32_t r[2][8];
+                for (int x0 = 0; x0 < H; x0 += XCH) {
+                    uint32_t hi[XCH], lo[XCH], m1[XCH];
 #pragma unroll
-                for (int qp = 0; qp < 2; ++qp)       // columns 32 (2 h + q') + y
-                    tmem_ld8_nowait(lane_base + 128u * (uint32_t)e + (uint32_t)(SL * (2 * h + qp) + 8 * yc), r[qp]);
-                ulonglong2 ep[4];
+                    for (int i = 0; i < XCH; i += 2) {
+                        const ulonglong2 e = *(const ulonglong2 *)(xs + (x0 + i) / 2);
+                        float ph[2];
+                        f2_unpack(f2_fma(cc2, e.y, f2_mul(ca2, e.x)), ph[0], ph[1]);
 #pragma unroll
-                for (int pp = 0; pp < 4; ++pp) ep[pp] = ey[(4 * yc + pp) * TV + kl];
-#pragma unroll
-                for (int qp = 0; qp < 2; ++qp) {
-                    tmem_wait_ld8(r[qp]);
-#pragma unroll
-                    for (int pp = 0; pp < 4; ++pp) {
-                        const f2_t v = f2_pack(__uint_as_float(r[qp][2 * pp]), __uint_as_float(r[qp][2 * pp + 1]));
-                        accp[qp][0] = f2_fma(ep[pp].x, v, accp[qp][0]);
-                        accp[qp][1] = f2_fma(ep[pp].y, v, accp[qp][1]);
+                        for (int j = 0; j < 2; ++j) {
+                            float sn, cs, m0, m2;
+                            __sincosf(ph[j], &sn, &cs);
+                            split_e(cs, sn, hi[i + j], lo[i + j]);
+                            f2_unpack(f2_mul(f2_pack(sn, cs), cz2), m0, m2);
+                            m1[i + j] = pack_f16x2(m0, m2);
+                        }
                     }
+                    const uint32_t ta = lane_base + C::A_COL + (uint32_t)(half * H + x0);
+                    tmem_st(ta, hi);
+                    tmem_st(ta + SL, lo);
+                    tmem_st(ta + 2 * SL, m1);
                 }
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
             }
-            float acc[2][2];
-#pragma unroll
-            for (int q2 = 0; q2 < 2; ++q2)
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    float lo, hi;
-                    f2_unpack(accp[q2][c], lo, hi);
-                    acc[q2][c] = lo + hi;
-                }
-            const float4 cfk = s_coef[e * TV + kl];
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(smem_u32(&s_dempty[e]));
-                mbar_arrive(smem_u32(&s_eyempty[e]));
-            }
-            // exchange with the other row of the visibility: the re row holds (er Tr, ei Tr),
-            // the im row (er Ti, ei Ti); Re(E T) = er Tr - ei Ti, Im(E T) = er Ti + ei Tr
-            float *part = s_part + (size_t)(s * 2 + ci) * (2 * 4 * TV) + (size_t)h * 4 * TV;
+            if (lane == 0) mbar_arrive(smem_u32(&s_afull));
+            if (t > 0) finish(t - 1);      // every warp was active in the tile before
+            // Ey* of this half's y, as pairs (cs_y, cs_y+1), (sn_y, sn_y+1), while the MMAs run
+            f2_t ec[H / 2], es[H / 2];
+            if (active) {
+                const f2_t cb2 = f2_pack(cb, cb), cc2 = f2_pack(cc, cc);
 #pragma unroll
-            for (int q2 = 0; q2 < 2; ++q2) {
-                part[(2 * q2) * TV + kl] = acc[q2][0];
-                part[(2 * q2 + 1) * TV + kl] = acc[q2][1];
+                for (int j = 0; j < H / 2; ++j) {
+                    const ulonglong2 e = *(const ulonglong2 *)(yt + j);
+                    float p0, p1, s0, c0, s1, c1;
+                    f2_unpack(f2_fma(cc2, e.y, f2_mul(cb2, e.x)), p0, p1);
+                    __sincosf(p0, &s0, &c0);
+                    __sincosf(p1, &s1, &c1);
+                    ec[j] = f2_pack(c0, c1);
+                    es[j] = f2_pack(s0, s1);
+                }
             }
-            consumers_sync();
-            const float *other = s_part + (size_t)(s * 2 + (ci ^ 1)) * (2 * 4 * TV) + (size_t)h * 4 * TV;
-            // this thread writes polarisation q' = ci of the pair
-            const int qp = ci;
-            const float own0 = ci ? acc[1][0] : acc[0][0];
-            const float own1 = ci ? acc[1][1] : acc[0][1];
-            const float oth0 = other[(2 * qp) * TV + kl], oth1 = other[(2 * qp + 1) * TV + kl];
-            const float a0 = ci ? oth0 : own0, a1 = ci ? oth1 : own1;     // er Tr, ei Tr
-            const float b0 = ci ? own0 : oth0, b1 = ci ? own1 : oth1;     // er Ti, ei Ti
-            const uint32_t vw = __float_as_uint(cfk.w);       // index (< 2^31 - 1), bit 31 = flagged
-            if (!(vw & 0x80000000u) && !failed) {
-                ((float2 *)vis_out)[4 * (size_t)vw + 2 * h + qp] = make_float2((a0 - b1) * inv_scale, (b0 + a1) * inv_scale);
-            } else if (vw != 0xFFFFFFFFu && !failed) {
-                ((float2 *)vis_out)[4 * (size_t)(vw & 0x7FFFFFFFu) + 2 * h + qp] = make_float2(0.f, 0.f);   // flagged
+            ovi = vi;
+            float acc[4][2];
+#pragma unroll
+            for (int p = 0; p < C::PARTS; ++p) {
+                if (p == C::PARTS - 1 && t + 1 < n_tiles) {
+                    form_coef(ca, cb, cc, vi);
+                    load_raw((t + 2) * TV + row);
+                }
+                wait_or_fail(smem_u32(&s_dfull), (uint32_t)((t * C::PARTS + p) & 1), failed);
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                if (active) {
+                    // y_q = sum_y (cs - i sn) T_q(y): Re = sum cs Tr + sn Ti, Im = sum cs Ti - sn Tr
+#pragma unroll
+                    for (int qp = 0; qp < QH; qp += 2) {
+                        f2_t re[2], ip[2], im[2];
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) re[e] = ip[e] = im[e] = 0ull;
+#pragma unroll
+                        for (int yc = 0; yc < H / YB; ++yc) {
+                            uint32_t r[2][2 * YB];
+#pragma unroll
+                            for (int e = 0; e < 2; ++e)
+                                tmem_ld_nowait(lane_base + (uint32_t)(2 * SL * (qp + e) + half * SL + 2 * YB * yc), r[e]);
+#pragma unroll
+                            for (int e = 0; e < 2; ++e) tmem_wait_ld(r[e]);
+#pragma unroll
+                            for (int e = 0; e < 2; ++e)
+#pragma unroll
+                                for (int j = 0; j < YB / 2; ++j) {
+                                    const f2_t Tr = f2_pack(__uint_as_float(r[e][2 * j]), __uint_as_float(r[e][2 * j + 1]));
+                                    const f2_t Ti = f2_pack(__uint_as_float(r[e][YB + 2 * j]),
+                                                            __uint_as_float(r[e][YB + 2 * j + 1]));
+                                    const f2_t c2 = ec[YB / 2 * yc + j], s2 = es[YB / 2 * yc + j];
+                                    re[e] = f2_fma(c2, Tr, re[e]);
+                                    ip[e] = f2_fma(c2, Ti, ip[e]);
+                                    im[e] = f2_fma(s2, Tr, im[e]);
+                                    re[e] = f2_fma(s2, Ti, re[e]);
+                                }
+                        }
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            float a0, a1, b0, b1, c0, c1;
+                            f2_unpack(re[e], a0, a1);
+                            f2_unpack(ip[e], b0, b1);
+                            f2_unpack(im[e], c0, c1);
+                            acc[p * QH + qp + e][0] = a0 + a1;
+                            acc[p * QH + qp + e][1] = (b0 + b1) - (c0 + c1);
+                        }
+                    }
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&s_dempty));
+            }
+            if (active) {
+                s_part[((t & 1) * 2 + (half ^ 1)) * TV + row] =
+                    half ? make_float4(acc[0][0], acc[0][1], acc[1][0], acc[1][1])
+                         : make_float4(acc[2][0], acc[2][1], acc[3][0], acc[3][1]);
+                own = half ? make_float4(acc[2][0], acc[2][1], acc[3][0], acc[3][1])
+                           : make_float4(acc[0][0], acc[0][1], acc[1][0], acc[1][1]);
             }
         }
+        if (n_tiles > 0 && (n_tiles - 1) * TV + 32 * quarter < kp) finish(n_tiles - 1);
         if (failed && lane == 0) atomicExch(&g_sepd_error, 1);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == MMA_WARP) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "n"(512));
+    if (warp == MMA_WARP)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "n"(TMEM_COLS));
 }
 
 // one CTA per subgrid of one plan (plan index idx[b] or first + b; image b of sub)
 template <int L>
-__global__ void __launch_bounds__(NT, 1)
+__global__ void __launch_bounds__(NT, CTAS)
 degridder_sep_kernel(Geometry g, const int32_t *__restrict__ idx, int64_t first, const float4 *__restrict__ sub,
                      const uint8_t *__restrict__ flags, const float4 *__restrict__ aterms,
                      const float *__restrict__ taper, float4 *__restrict__ vis_out) {
@@ -551,7 +493,7 @@ degridder_sep_kernel(Geometry g, const int32_t *__restrict__ idx, int64_t first,
 
 // fused: one CTA per subgrid, read from the grid
 template <int L>
-__global__ void __launch_bounds__(NT, 1)
+__global__ void __launch_bounds__(NT, CTAS)
 degridder_sep_fused_kernel(Geometry g, const int32_t *__restrict__ idx, int64_t first, const float4 *__restrict__ grid,
                            const uint8_t *__restrict__ flags, const float4 *__restrict__ aterms,
                            const float *__restrict__ taper, float4 *__restrict__ vis_out) {
