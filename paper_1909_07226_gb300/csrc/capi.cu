@@ -247,6 +247,8 @@ idg::Geometry idg_plan::geometry() const {
     g.scale_f2 = d_scale_f2;
     g.nprime = d_nprime;
     g.sep = d_nprime + (size_t)L * L;
+    std::copy(sep_s, sep_s + 32, g.sep_s);
+    std::copy(sep_t, sep_t + 32, g.sep_t);
     g.separable = stats.separable;
     g.c_scale = c_scale;
     g.r_scale = r_scale;
@@ -751,6 +753,10 @@ idg_status idg_plan_create(const double *uvw_m, const double *freqs_hz, const in
     for (int i = 0; i < L; ++i) {
         nprime[(size_t)L * L + i] = (float)n1(i, j0);
         nprime[(size_t)L * L + L + i] = (float)(n1(j0, i) - n1(j0, j0));
+        if (i < 32) {
+            p->sep_s[i] = nprime[(size_t)L * L + i];
+            p->sep_t[i] = nprime[(size_t)L * L + L + i];
+        }
     }
 
     // the default taper (calls with a NULL taper): c[y][x] = a_y a_x with a the PSWF

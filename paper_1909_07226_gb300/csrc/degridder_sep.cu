@@ -80,8 +80,7 @@ struct SepD {
     // prologue scratch over B: the subgrid's grid rows, then the transform planes
     static constexpr int FFT_P = L + 1, FFT_OFF = SPIX * 32, FFT_BYTES = 4 * L * FFT_P * 8;
     static constexpr int PART_OFF = B_BYTES > FFT_OFF + FFT_BYTES ? B_BYTES : FFT_OFF + FFT_BYTES;
-    static constexpr int SEP_OFF = PART_OFF + 2 * 2 * TV * 16;   // [2 tiles][2 pol pairs][TV] float4 (y halves meet)
-    static constexpr int SMEM = SEP_OFF + 2 * (L / 2) * 16;      // (X, X + 1, s(X), s(X + 1)) per x pair, t alike
+    static constexpr int SMEM = PART_OFF + 2 * 2 * TV * 16;      // [2 tiles][2 pol pairs][TV] float4 (y halves meet)
     // tensor memory: accumulator, then A hi, lo and m = 1, one column per x
     static constexpr uint32_t A_COL = PN;
     static constexpr uint32_t IDESC = idesc_m128(PN);
@@ -108,6 +107,54 @@ __device__ __forceinline__ void pair_sync(int quarter) {
     }
 }
 
+// A of a visibility's x from X0: (cs, sn) of Ex, its FP16 hi and lo parts and the m = 1 factor,
+// into its tensor-memory row.  X and s(x) are instruction constants (kernel parameters), so
+// the loop reads no memory.
+template <int L, int X0>
+__device__ __forceinline__ void form_a(const Geometry &g, uint32_t lane_base, float csig, float ca, float cc) {
+    using C = SepD<L>;
+    constexpr int SL = L, H = C::H, XCH = C::XCH;
+    constexpr float magic_1 = 6144.0f;      // split at multiples of 2^-11
+    const float cz = cc * csig;
+    const f2_t cz2 = f2_pack(cz, cz), nz2 = f2_pack(-cz, -cz);
+#pragma unroll
+        for (int x0 = X0; x0 < X0 + H; x0 += XCH) {
+            uint32_t hi[XCH], lo[XCH], m1[XCH];
+#pragma unroll
+            for (int i = 0; i < XCH; i += 2) {
+                float sn0, cs0, sn1, cs1;
+                __sincosf(fmaf(cc, g.sep_s[x0 + i], ca * (float)(x0 + i - SL / 2)), &sn0, &cs0);
+                __sincosf(fmaf(cc, g.sep_s[x0 + i + 1], ca * (float)(x0 + i + 1 - SL / 2)), &sn1, &cs1);
+                const f2_t c2 = f2_pack(cs0, cs1), s2 = f2_pack(sn0, sn1);
+                f2_t hc, lc, hs, ls;
+                f2_split(c2, magic_1, hc, lc);
+                f2_split(s2, magic_1, hs, ls);
+                pack_pairs(hc, hs, hi[i], hi[i + 1]);
+                pack_pairs(lc, ls, lo[i], lo[i + 1]);
+                pack_pairs(f2_mul(nz2, s2), f2_mul(cz2, c2), m1[i], m1[i + 1]);
+            }
+            const uint32_t ta = lane_base + C::A_COL + (uint32_t)x0;
+            tmem_st(ta, hi);
+            tmem_st(ta + SL, lo);
+            tmem_st(ta + 2 * SL, m1);
+        }
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+
+// Ey* of its y from Y0 as pairs (cs_y, cs_y+1), (sn_y, sn_y+1)
+template <int L, int Y0>
+__device__ __forceinline__ void form_ey(const Geometry &g, float cb, float cc, f2_t (&ec)[L / 4], f2_t (&es)[L / 4]) {
+    constexpr int SL = L, H = L / 2;
+#pragma unroll
+        for (int j = 0; j < H / 2; ++j) {
+            float s0, c0, s1, c1;
+            __sincosf(fmaf(cc, g.sep_t[Y0 + 2 * j], cb * (float)(Y0 + 2 * j - SL / 2)), &s0, &c0);
+            __sincosf(fmaf(cc, g.sep_t[Y0 + 2 * j + 1], cb * (float)(Y0 + 2 * j + 1 - SL / 2)), &s1, &c1);
+            ec[j] = f2_pack(c0, c1);
+            es[j] = f2_pack(s0, s1);
+        }
+}
+
 // Visibilities of subgrid d of geometry g from its image src[L][L][4], or with
 // FUSED from the grid src[layer][N][N][4]: split and transformed in shared memory
 // first (Algorithm 2: split from the master grid, "IFFT", image-domain kernel, sum).
@@ -121,7 +168,6 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
     extern __shared__ __align__(1024) uint8_t smem[];
     float2 *s_fft = (float2 *)(smem + C::FFT_OFF);       // [4][L][L + 1] during the prologue
     float4 *s_part = (float4 *)(smem + C::PART_OFF);
-    float4 *s_sep = (float4 *)(smem + C::SEP_OFF);       // x pairs, then y pairs
     __shared__ uint32_t s_tmem;
     __shared__ __align__(8) uint64_t s_afull, s_dfull, s_dempty, s_drain, s_gbar;
     __shared__ float s_red[NWW];
@@ -152,10 +198,6 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
             bulk_g2s(smem_u32(smem + lane * SL * 32), gsrc + 2 * ((size_t)(d.r0 + lane) * g.N + d.q0), SL * 32,
                      smem_u32(&s_gbar));
         }
-    }
-    if (tid < SL) {
-        const float X = (float)((2 * tid) % SL - SL / 2);
-        s_sep[tid] = make_float4(X, X + 1.0f, g.sep[2 * tid], g.sep[2 * tid + 1]);
     }
 
     // workers: visibility 32 (warp % 4) + lane of the tile, x and y half warp / 4
@@ -329,7 +371,6 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
     } else {
         const uint32_t lane_base = tmem + ((uint32_t)(32 * quarter) << 16);
         const float csig = g.c_scale;
-        const float4 *xs = s_sep + half * (H / 2), *yt = s_sep + (SL + half * H) / 2;
         // phase coefficients of the tile's visibility from float pairs (error-free products and
         // sums, rounded once), and its output index; formed one tile ahead, while MMAs run
         float ca = 0.f, cb = 0.f, cc = 0.f;
@@ -364,32 +405,8 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
             // A: this half's x of the visibility's row (the last part of the previous tile was waited
             // for below, so the MMAs are done with A)
             if (active) {
-                const float cz = cc * csig;
-                const f2_t ca2 = f2_pack(ca, ca), cc2 = f2_pack(cc, cc), cz2 = f2_pack(-cz, cz);
-                constexpr int XCH = C::XCH;
-#pragma unroll 1
-                for (int x0 = 0; x0 < H; x0 += XCH) {
-                    uint32_t hi[XCH], lo[XCH], m1[XCH];
-#pragma unroll
-                    for (int i = 0; i < XCH; i += 2) {
-                        const ulonglong2 e = *(const ulonglong2 *)(xs + (x0 + i) / 2);
-                        float ph[2];
-                        f2_unpack(f2_fma(cc2, e.y, f2_mul(ca2, e.x)), ph[0], ph[1]);
-#pragma unroll
-                        for (int j = 0; j < 2; ++j) {
-                            float sn, cs, m0, m2;
-                            __sincosf(ph[j], &sn, &cs);
-                            split_e(cs, sn, hi[i + j], lo[i + j]);
-                            f2_unpack(f2_mul(f2_pack(sn, cs), cz2), m0, m2);
-                            m1[i + j] = pack_f16x2(m0, m2);
-                        }
-                    }
-                    const uint32_t ta = lane_base + C::A_COL + (uint32_t)(half * H + x0);
-                    tmem_st(ta, hi);
-                    tmem_st(ta + SL, lo);
-                    tmem_st(ta + 2 * SL, m1);
-                }
-                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                if (half) form_a<L, H>(g, lane_base, csig, ca, cc);
+                else form_a<L, 0>(g, lane_base, csig, ca, cc);
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
@@ -398,17 +415,8 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
             // Ey* of this half's y, as pairs (cs_y, cs_y+1), (sn_y, sn_y+1), while the MMAs run
             f2_t ec[H / 2], es[H / 2];
             if (active) {
-                const f2_t cb2 = f2_pack(cb, cb), cc2 = f2_pack(cc, cc);
-#pragma unroll
-                for (int j = 0; j < H / 2; ++j) {
-                    const ulonglong2 e = *(const ulonglong2 *)(yt + j);
-                    float p0, p1, s0, c0, s1, c1;
-                    f2_unpack(f2_fma(cc2, e.y, f2_mul(cb2, e.x)), p0, p1);
-                    __sincosf(p0, &s0, &c0);
-                    __sincosf(p1, &s1, &c1);
-                    ec[j] = f2_pack(c0, c1);
-                    es[j] = f2_pack(s0, s1);
-                }
+                if (half) form_ey<L, H>(g, cb, cc, ec, es);
+                else form_ey<L, 0>(g, cb, cc, ec, es);
             }
             ovi = vi;
             float acc[4][2];

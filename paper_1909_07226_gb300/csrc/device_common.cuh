@@ -158,10 +158,23 @@ __device__ __forceinline__ f2_t f2_fma(f2_t a, f2_t b, f2_t c) {
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
     return d;
 }
+__device__ __forceinline__ f2_t f2_add(f2_t a, f2_t b) {
+    f2_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
 __device__ __forceinline__ f2_t f2_mul(f2_t a, f2_t b) {
     f2_t d;
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
+}
+__device__ __forceinline__ f2_t f2_bcast(float v) { return f2_pack(v, v); }
+// v = hi + lo with hi the multiple of ulp(magic) nearest to v (magic = 1.5 x a power of two far
+// above |v|): exact.  For |v| <= 2048 ulp(magic), hi fits FP16 exactly, and lo, at most half
+// that ulp, is rounded by its own FP16 conversion at 2^-12 of itself.
+__device__ __forceinline__ void f2_split(f2_t v, float magic, f2_t &hi, f2_t &lo) {
+    hi = f2_add(f2_add(v, f2_bcast(magic)), f2_bcast(-magic));
+    lo = f2_fma(hi, f2_bcast(-1.0f), v);
 }
 
 // ---------------------------------------------------------------------------

@@ -73,51 +73,47 @@ namespace {
 using namespace dev;
 using namespace tc;
 
-constexpr int NPW = 16;                        // producer warps
+constexpr int NPW = 8;                         // producer warps: two sets of four
 constexpr int NP = NPW * 32;                   // producer threads
 constexpr int NT = NP + 32;                    // + the MMA warp
+constexpr int CTAS = 2;                        // per SM
 constexpr int VB = NP;                         // visibilities per staged batch (one per producer)
-constexpr int GB = VB / 8;                     // groups per batch
-constexpr int FOLD = 64;                       // groups per accumulation period
-constexpr int SG = 8;                          // groups of 8 visibilities per stage
-constexpr int STAGES = 2;
-static_assert(FOLD / SG >= STAGES, "a period spans at least STAGES stages");
-static_assert((STAGES & (STAGES - 1)) == 0, "STAGES is a power of two");
-static_assert(FOLD % SG == 0 && GB % SG == 0, "periods and batches are whole stages");
+constexpr int SG = 2;                          // groups of 8 visibilities per stage
+constexpr int SPB = VB / (8 * SG);             // stages per batch
+constexpr int SPP = 2 * SPB;                   // stages per accumulation period (512 visibilities)
+constexpr uint32_t TMEM_COLS = 256;            // two CTAs share an SM's 512
 
 // Layout for subgrid size L (32, 24 or 16).  A has 128 rows: lane quarter yq holds pixel
-// rows y = (L / 4) yq + ylo for ylo < L / 4 at lanes 8 q + ylo (lanes with ylo >= L / 4
-// carry zeros: ylo = 6, 7 at L = 24, ylo >= 4 at L = 16).  B has 6 L rows per group: (m = 0, re), (m = 0, im), (m = 1, re),
-// (m = 1, im), then the lo parts of m = 0 re and im, L rows each.
+// rows y = 8 yq + ylo at lanes 8 q + ylo (quarters from L / 8 on are not used: their rows of
+// the accumulator are never read).  B has 6 L rows per group: (m = 0, re), (m = 0, im),
+// (m = 1, re), (m = 1, im), then the lo parts of m = 0 re and im, L rows each.
 template <int L>
 struct SepG {
-    static constexpr int SL = L, SPIX = L * L, YQ = L / 4;
+    static constexpr int SL = L, SPIX = L * L, NQ = L / 8;   // NQ: 8-row (and 8-column) blocks
     static constexpr int B_GROUP = 6 * L * 32;   // B of one group: 6 L rows x 16 K FP16
     static constexpr int B_STAGE = SG * B_GROUP;
-    // coefficients as two float pairs, [2][VB] (b, c) for the Ey side, then [2][VB] (a, c)
-    // for the Ex side: the shared-memory pipe is close to its limit in the main loop and its
-    // cost is the bytes each thread reads (a float4 where two floats are used costs twice)
-    static constexpr int COEF_OFF = STAGES * B_STAGE;
-    static constexpr int VIS_OFF = COEF_OFF + 2 * VB * 16;   // [2][VB][4] float2 (scaled V)
-    static constexpr int FOLD_OFF = VIS_OFF + 2 * VB * 32;   // [32][NP] float: folded sums of each producer
-    static constexpr int SMEM = FOLD_OFF + 32 * NP * 4;
-    static constexpr int FFT_P = L + 1;
-    // the subgrid's A-terms after the main loop: [2 stations][L^2] 2 x 2 complex, beside the
-    // transform planes, over the stage and coefficient buffers
-    static constexpr int AT_OFF = 4 * L * FFT_P * 8;
+    // the subgrid image (polarisation planes, row pitch L + 1): the folded sums, then transformed in place
+    static constexpr int FFT_P = L + 1, IMG_BYTES = 4 * L * FFT_P * 8;
+    static constexpr int B_OFF = IMG_BYTES;      // [2 sets][2 buffers][SG groups]
+    // staged batches, [2] each, visibility pairs: (b0, b1, c0, c1), (a0, a1, c0, c1) and per
+    // polarisation (re0, re1, im0, im1)
+    static constexpr int CB_OFF = B_OFF + 4 * B_STAGE, CA_OFF = CB_OFF + 2 * VB * 8;
+    static constexpr int VIS_OFF = CA_OFF + 2 * VB * 8;
+    static constexpr int SMEM = VIS_OFF + 2 * VB * 32;
+    // the subgrid's A-terms after the main loop: [2 stations][L^2] 2 x 2 complex, over B and the batches
+    static constexpr int AT_OFF = B_OFF;
     static constexpr uint32_t AT_BYTES = SPIX * 32;
     // accumulator: main (m, re/im, x) at 0 .. 4 L, correction (m = 0) at 4 L .. 6 L; then the
-    // A stages
+    // sets' A, 32 columns each (group i at + 16 i: 8 columns hi, 8 lo)
     static constexpr uint32_t A_COL = 6 * L;
     static constexpr uint32_t IDESC_NB = idesc_m128(6 * L), IDESC_NC = idesc_m128(2 * L);
-    static constexpr int NSL = L / 8;             // 16-column slices of the m = 0 block (fold)
-    static constexpr int XS = L / 4;              // x values per producer in the epilogue
+    static constexpr int XS = L / 2, XC = 4;               // x per set in the fold, in chunks
+    static constexpr int PIXT = (SPIX + NP - 1) / NP;            // pixels per producer in the epilogue
     static_assert(L == 32 || L == 24 || L == 16, "subgrid sizes of the separable kernels");
-    static_assert(4 * L * FFT_P * 8 <= FOLD_OFF, "transform planes fit over the stage buffers");
-    static_assert(SMEM + 1024 <= 227 * 1024, "dynamic and static shared memory of one CTA");
-    static_assert(AT_OFF % 16 == 0 && AT_OFF + 2 * (int)AT_BYTES <= VIS_OFF, "A-terms over the stage and coefficient buffers");
-    static_assert(A_COL % 16 == 0 && A_COL + 16 * SG * STAGES <= 512, "tensor memory");
-    static_assert(NSL <= NPW / 4, "one fold slice per warp of a lane quarter");
+    static_assert(CTAS * (SMEM + 2048) <= 227 * 1024, "shared memory of the SM's CTAs");
+    static_assert(AT_OFF % 16 == 0 && AT_OFF + 2 * (int)AT_BYTES <= SMEM, "A-terms over B and the batches");
+    static_assert(B_OFF % 128 == 0 && CB_OFF % 16 == 0, "alignment of the B tiles and the batches");
+    static_assert(A_COL % 16 == 0 && A_COL + 2 * 16 * SG <= TMEM_COLS, "tensor memory");
 };
 
 __device__ __forceinline__ void producers_sync() { asm volatile("bar.sync 1, %0;" :: "n"(NP) : "memory"); }
@@ -131,25 +127,23 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
                                                  const float4 *__restrict__ aterms, const float *__restrict__ taper,
                                                  float4 *__restrict__ o) {
     using C = SepG<L>;
-    constexpr int SL = C::SL, SPIX = C::SPIX, YQ = C::YQ, B_GROUP = C::B_GROUP, B_STAGE = C::B_STAGE;
-    constexpr int COEF_OFF = C::COEF_OFF, VIS_OFF = C::VIS_OFF, FOLD_OFF = C::FOLD_OFF, FFT_P = C::FFT_P;
-    constexpr int AT_OFF = C::AT_OFF, XS = C::XS;
+    constexpr int SL = C::SL, SPIX = C::SPIX, NQ = C::NQ, B_GROUP = C::B_GROUP, B_STAGE = C::B_STAGE;
+    constexpr int FFT_P = C::FFT_P, AT_OFF = C::AT_OFF, XS = C::XS, PIXT = C::PIXT;
     constexpr uint32_t AT_BYTES = C::AT_BYTES, A_COL = C::A_COL;
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint8_t *sB = smem;
-    float2 *s_cb = (float2 *)(smem + COEF_OFF);          // [2][VB] (b, c)
-    float2 *s_ca = s_cb + 2 * VB;                         // [2][VB] (a, c)
-    float2 *s_vis = (float2 *)(smem + VIS_OFF);
-    float2 *s_fft = (float2 *)smem;                 // [4][L][L + 1] after the main loop
-    float *s_fold = (float *)(smem + FOLD_OFF);     // [32][NP]: m = 0 sums (16), then m = 1 (16)
+    float2 *s_img = (float2 *)smem;                 // [4][L][L + 1]
+    uint8_t *sB = smem + C::B_OFF;
+    float *s_cb = (float *)(smem + C::CB_OFF), *s_ca = (float *)(smem + C::CA_OFF);
+    float *s_vis = (float *)(smem + C::VIS_OFF);
     __shared__ uint32_t s_tmem;
-    __shared__ __align__(8) uint64_t s_full[STAGES], s_empty[STAGES], s_foldbar, s_folded, s_drain, s_atbar;
-    __shared__ float s_red[2][NPW];
+    __shared__ __align__(8) uint64_t s_full[2], s_empty[2], s_foldbar, s_folded, s_drain, s_atbar;
+    __shared__ float s_red[NPW];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool mma_warp = warp == NPW;
-    const int total_groups = (d.kp + 7) / 8;
-    const int n_batches = (d.kp + VB - 1) / VB;     // = accumulation periods (FOLD = GB)
+    const int kp = d.kp;
+    const int total_groups = (kp + 7) / 8, n_stages = (total_groups + SG - 1) / SG;
+    const int n_batches = (kp + VB - 1) / VB, n_periods = (n_stages + SPP - 1) / SPP;
 
     // staging (producers): visibility tid of batch b, loaded into registers one batch ahead;
     // the first batch's loads go out before the set-up below, so their latency overlaps it
@@ -158,33 +152,67 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
     bool pin = false, pflag = false;
     const float4 *uvw2 = (const float4 *)g.uvw_f2;
     const float4 *sc2 = (const float4 *)g.scale_f2;
+    const size_t bt0 = (size_t)d.bl * g.n_t + d.t0;
+    const int dt = VB / d.nc, dc = VB - dt * d.nc;     // a batch's step in timestep and channel
+    const int vt0 = tid / d.nc, vc0 = tid - vt0 * d.nc;
+    int vt = vt0, vc = vc0;
+    auto advance = [&](int &t, int &c) {
+        t += dt;
+        c += dc;
+        if (c >= d.nc) {
+            c -= d.nc;
+            ++t;
+        }
+    };
     auto load_batch = [&](int b) {
-        const int k = b * VB + tid;
-        pin = k < d.kp;
+        pin = b * VB + tid < kp;
         pflag = false;
         if (pin) {
-            int t, c;
-            const size_t vi = vis_index(g, d, k, t, c);
-            const size_t bt = (size_t)d.bl * g.n_t + t;
+            const size_t bt = bt0 + vt;
+            const int c = d.c0 + vc;
+            const size_t vi = bt * g.n_chan + c;
             puv = uvw2[2 * bt];
-            const float4 w4 = uvw2[2 * bt + 1];
-            pw = make_float2(w4.x, w4.y);
+            pw = *(const float2 *)(uvw2 + 2 * bt + 1);
             pws = sc2[c];
             pflag = flags && flags[vi];
             pa = vis[2 * vi];          // loaded whatever the flag: the load does not wait for it
             pb = vis[2 * vi + 1];
         }
+        advance(vt, vc);
+    };
+    auto max_of = [](const float4 &a, const float4 &b) {
+        return fmaxf(fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(a.z), fabsf(a.w))),
+                     fmaxf(fmaxf(fabsf(b.x), fabsf(b.y)), fmaxf(fabsf(b.z), fabsf(b.w))));
     };
     if (!mma_warp) load_batch(0);
 
     if (mma_warp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     :: "r"(smem_u32(&s_tmem)), "n"(512));
+                     :: "r"(smem_u32(&s_tmem)), "n"(TMEM_COLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    } else {
+        // the subgrid's largest unflagged |component| (the visibilities past the first batch are
+        // read here once more, for the scale; they come back from L2 when they are staged)
+        float m = 0.0f;
+        {
+            int t = vt0, c = vc0;
+            advance(t, c);
+#pragma unroll 4
+            for (int k = VB + tid; k < kp; k += VB) {
+                const size_t vi = (bt0 + t) * g.n_chan + d.c0 + c;
+                const float mk = max_of(vis[2 * vi], vis[2 * vi + 1]);
+                if (!(flags && flags[vi])) m = fmaxf(m, mk);
+                advance(t, c);
+            }
+        }
+        if (pin && !pflag) m = fmaxf(m, max_of(pa, pb));
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+        if (lane == 0) s_red[warp] = m;
     }
     if (tid == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            mbar_init(smem_u32(&s_full[s]), NPW);
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(smem_u32(&s_full[s]), NPW / 2);
             mbar_init(smem_u32(&s_empty[s]), 1);
         }
         mbar_init(smem_u32(&s_foldbar), 1);
@@ -199,51 +227,41 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
     const uint32_t tmem = s_tmem;
 
     bool failed = false, at_issued = false;
-    // the taper of this thread's epilogue pixels, loaded at the end of its main loop
-    constexpr int NPIX = (SPIX + NT - 1) / NT;
-    float tw_pre[NPIX];
-    auto load_taper = [&]() {
-#pragma unroll
-        for (int i = 0; i < NPIX; ++i) tw_pre[i] = tid + i * NT < SPIX ? taper[tid + i * NT] : 0.0f;
-    };
-    const int yq = warp & 3, sl = warp >> 2;        // lane quarter (rows 32 yq ..) and fold column slice
+    const int yq = warp & 3, set = (warp >> 2) & 1;   // lane quarter (rows 32 yq ..) and producer set
 
     if (mma_warp) {
         if (lane == 0) {
-            // descriptors and tensor-memory addresses advance by constants: stage s, group i at
-            // B + s B_STAGE + i B_GROUP (the descriptor's address field counts 16-byte units)
+            // descriptors and tensor-memory addresses advance by constants (the descriptor's
+            // address field counts 16-byte units)
             const uint64_t db0 = smem_desc(smem_u32(sB));
-            const int n_stages = (total_groups + SG - 1) / SG;
-            constexpr int SPP = FOLD / SG;                  // stages per accumulation period
             for (int st = 0; st < n_stages; ++st) {
-                const int s = st & (STAGES - 1);
+                const int s = st & 1, use = st >> 1;        // set, and its how manieth stage
                 const bool first = st % SPP == 0, last = st % SPP == SPP - 1 || st == n_stages - 1;
                 if (first && st > 0) {         // the producers have read the previous period
                     wait_or_fail(smem_u32(&s_folded), (uint32_t)(((st / SPP) - 1) & 1), failed);
                 }
-                wait_or_fail(smem_u32(&s_full[s]), (uint32_t)((st / STAGES) & 1), failed);
+                wait_or_fail(smem_u32(&s_full[s]), (uint32_t)(use & 1), failed);
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const int ng = min(SG, total_groups - st * SG);
-                const uint64_t dbs = db0 + (uint64_t)((s * B_STAGE) >> 4);
+                const uint64_t dbs = db0 + (uint64_t)(((2 * s + (use & 1)) * B_STAGE) >> 4);
                 const uint32_t ats = tmem + A_COL + 16u * SG * (uint32_t)s;
 #pragma unroll
                 for (int i = 0; i < SG; ++i) {
                     if (i < ng) {
-                        mma_ta_i(tmem, ats + 16u * i, dbs + (uint64_t)((i * B_GROUP) >> 4), C::IDESC_NB,
-                                 (first && i == 0) ? 0u : 1u);
-                        mma_ta_i(tmem + 4u * SL, ats + 16u * i + 8u, dbs + (uint64_t)((i * B_GROUP) >> 4), C::IDESC_NC,
-                                 1u);
+                        const uint64_t db = dbs + (uint64_t)((i * B_GROUP) >> 4);
+                        mma_ta_i(tmem, ats + 16u * i, db, C::IDESC_NB, (first && i == 0) ? 0u : 1u);
+                        mma_ta_i(tmem + 4u * SL, ats + 16u * i + 8u, db, C::IDESC_NC, 1u);
                     }
                 }
-                if (last) commit(smem_u32(&s_foldbar));
                 commit(smem_u32(&s_empty[s]));
+                if (last) commit(smem_u32(&s_foldbar));
             }
             commit(smem_u32(&s_drain));
             bool late = false;
             wait_or_fail(smem_u32(&s_drain), 0u, late);     // bounded: let own MMAs finish before the free
             if (late) failed = true;
             // the tensor cores are done with the stage buffers: bring the subgrid's A-terms (A_p,
-            // A_q) into them while the producers fold and form the image
+            // A_q) into them while the producers fold
             if (aterms && !failed) {
                 const float4 *base = aterms + 2 * ((size_t)d.slot * g.n_stations) * SPIX;
                 mbar_expect_tx(smem_u32(&s_atbar), 2 * AT_BYTES);
@@ -254,227 +272,240 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
             }
         }
         failed = __shfl_sync(0xffffffffu, failed, 0);
-        load_taper();
     } else {
-        // A rows: r = 32 yq + lane holds polarisation qa = lane / 8 of pixel row y = YQ yq + lane % 8
-        // (rows with lane % 8 >= YQ are zero)
-        const int qa = lane >> 3, ylo = lane & 7;
-        const bool row_ok = YQ == 8 || ylo < YQ;
-        const int yrow = YQ * yq + (row_ok ? ylo : 0);
-        const int ga = warp >> 2;                   // group of the stage whose A entries this warp writes
-        const uint32_t lane_base = tmem + ((uint32_t)(32 * yq) << 16);
-        // Ey of row y for visibilities 2 qa and 2 qa + 1 of the group: computed here, shared by shuffles
-        const float Yv = (float)(yrow - SL / 2);
-        const float ty = g.sep[SL + yrow];
-        // B entries: x = 8 (warp & 3) + lane % 8, visibility j = 4 jh + lane / 8 of group i, where
-        // (i, jh) = (combo / 2, combo % 2) for combo = 2 (warp / 4) + t, t = 0, 1
-        const int xb = 8 * (warp & 3) + (lane & 7), jl = lane >> 3;
-        const bool x_ok = SL == 32 || xb < SL;      // the same for the whole warp (L is a multiple of 8)
-        const float Xv = (float)(xb - SL / 2);
-        const float sx = g.sep[x_ok ? xb : 0];
-        const float csig = g.c_scale;
-        const uint16_t m1h = 0xBC00u;      // FP16 -1
-
-        // phase coefficients of the staged visibility: u (f/c) k_uv - u0 k_uv and so on, from
-        // float pairs with error-free products and sums, rounded once to FP32
-        float4 cf_next = make_float4(0.f, 0.f, 0.f, 0.f);
-        auto form_coef = [&]() {
-            cf_next = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (pin) {
-                cf_next.x = pair_coef(puv.x, puv.y, pws.x, pws.y, d.a0h, d.a0l);
-                cf_next.y = pair_coef(puv.z, puv.w, pws.x, pws.y, d.b0h, d.b0l);
-                cf_next.z = pair_coef(pw.x, pw.y, pws.z, pws.w, d.csh, d.csl);
-            }
-        };
-        // coefficients and raw V of the batch; the batch's largest |component| into s_red[bb]
-        auto store_batch = [&](int bb) {
-            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-            if (pin && !pflag) {
-                a = pa;
-                b = pb;
-            }
-            s_cb[bb * VB + tid] = make_float2(cf_next.y, cf_next.z);
-            s_ca[bb * VB + tid] = make_float2(cf_next.x, cf_next.z);
-            float4 *dv = (float4 *)(s_vis + (size_t)(bb * VB + tid) * 4);
-            dv[0] = a;
-            dv[1] = b;
-            float m = fmaxf(fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(a.z), fabsf(a.w))),
-                            fmaxf(fmaxf(fabsf(b.x), fabsf(b.y)), fmaxf(fabsf(b.z), fabsf(b.w))));
+        // the subgrid's power-of-two scale: largest |component| of V in [2^9, 2^10)
+        float m = 0.0f;
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-            if (lane == 0) s_red[bb][warp] = m;
-        };
-        float inv_sc0 = 1.0f, inv_sc1 = 1.0f;        // 1 / scale of the last even and odd batch
+        for (int w = 0; w < NPW; ++w) m = fmaxf(m, s_red[w]);
+        int e2 = 0;
+        if (m > 0.0f) frexpf(m, &e2);
+        const float scale = ldexpf(1.0f, 10 - e2), inv_scale = ldexpf(1.0f, e2 - 10);
+        const uint32_t lane_base = tmem + ((uint32_t)(32 * yq) << 16);
+        const float csig = g.c_scale, rs = 1.0f / csig;
+        // FP16 hi/lo split points: A's |components| are below 2^10 sqrt(2) (integers fit FP16 up to
+        // 2^11), B's at most 1 (multiples of 2^-11)
+        constexpr float magic_a = 12582912.0f, magic_1 = 6144.0f;
 
+        // batch bb of the staged visibilities: phase coefficients u (f/c) k_uv - u0 k_uv and so on
+        // (float pairs, error-free products and sums, rounded once to FP32), scaled V (flagged: 0)
+        auto store_batch = [&](int bb) {
+            float ca = 0.f, cb = 0.f, cc = 0.f;
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+            if (pin) {
+                ca = pair_coef(puv.x, puv.y, pws.x, pws.y, d.a0h, d.a0l);
+                cb = pair_coef(puv.z, puv.w, pws.x, pws.y, d.b0h, d.b0l);
+                cc = pair_coef(pw.x, pw.y, pws.z, pws.w, d.csh, d.csl);
+                if (!pflag) {
+                    a = make_float4(pa.x * scale, pa.y * scale, pa.z * scale, pa.w * scale);
+                    b = make_float4(pb.x * scale, pb.y * scale, pb.z * scale, pb.w * scale);
+                }
+            }
+            const int at = bb * VB * 2 + (tid >> 1) * 4 + (tid & 1);
+            s_cb[at] = cb;
+            s_cb[at + 2] = cc;
+            s_ca[at] = ca;
+            s_ca[at + 2] = cc;
+            float *v = s_vis + bb * VB * 8 + (tid >> 1) * 4 + (tid & 1);     // [q][pair]
+            v[0] = a.x;
+            v[2] = a.y;
+            v[2 * VB] = a.z;
+            v[2 * VB + 2] = a.w;
+            v[4 * VB] = b.x;
+            v[4 * VB + 2] = b.y;
+            v[6 * VB] = b.z;
+            v[6 * VB + 2] = b.w;
+        };
+
+        // one period's accumulator, I = S0 + i r S1 / sigma of this thread's row (polarisation
+        // lane / 8, y = 8 yq + lane % 8) and its set's x, added to the image in FP32 (RN); the
+        // accumulator is released right after the loads
         auto fold = [&](int P) {
             wait_or_fail(smem_u32(&s_foldbar), (uint32_t)(P & 1), failed);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            // this thread's row, columns 16 sl .. of the m = 0 block (main + correction) and of m = 1;
-            // the accumulator is released right after the loads
-            constexpr bool all_fold = C::NSL == NPW / 4;
-            if (!all_fold && sl >= C::NSL) {      // no slice of the m = 0 block for this warp
+            constexpr int XC = C::XC;
+            if (yq < NQ) {
+                const int y = 8 * yq + (lane & 7);
+                float2 *img = s_img + ((lane >> 3) * SL + y) * FFT_P + set * XS;
+                const float *rp = g.sep + 2 * SL + y * SL + set * XS;
+#pragma unroll
+                for (int x0 = 0; x0 < XS; x0 += XC) {
+                    uint32_t re[XC], im[XC], cr[XC], ci[XC], r1[XC], i1[XC];
+                    const uint32_t base = lane_base + (uint32_t)(set * XS + x0);
+                    tmem_ld_nowait(base, re);
+                    tmem_ld_nowait(base + SL, im);
+                    tmem_ld_nowait(base + 2 * SL, r1);
+                    tmem_ld_nowait(base + 3 * SL, i1);
+                    tmem_ld_nowait(base + 4 * SL, cr);
+                    tmem_ld_nowait(base + 5 * SL, ci);
+                    tmem_wait_ld(re);
+                    tmem_wait_ld(im);
+                    tmem_wait_ld(r1);
+                    tmem_wait_ld(i1);
+                    tmem_wait_ld(cr);
+                    tmem_wait_ld(ci);
+                    if (x0 + XC == XS) {
+                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(&s_folded));
+                    }
+#pragma unroll
+                    for (int i = 0; i < XC; ++i) {
+                        const float rr = rp[x0 + i] * rs;
+                        const float vr = fmaf(-rr, __uint_as_float(i1[i]), __uint_as_float(re[i]) + __uint_as_float(cr[i]));
+                        const float vi = fmaf(rr, __uint_as_float(r1[i]), __uint_as_float(im[i]) + __uint_as_float(ci[i]));
+                        float2 f = P ? img[x0 + i] : make_float2(0.f, 0.f);
+                        img[x0 + i] = make_float2(fmaf(vr, inv_scale, f.x), fmaf(vi, inv_scale, f.y));
+                    }
+                }
+            } else {
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&s_folded));
-                return;
-            }
-            uint32_t r[16], rc[16], r1[16];
-            const uint32_t base = lane_base + 16u * (uint32_t)sl;
-            tmem_ld16(base, r);
-            tmem_ld16(base + 4u * SL, rc);
-            tmem_ld16(base + 2u * SL, r1);
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&s_folded));
-            const float is = (P & 1) ? inv_sc1 : inv_sc0;
-#pragma unroll
-            for (int c = 0; c < 16; ++c) {
-                const float v = (__uint_as_float(r[c]) + __uint_as_float(rc[c])) * is;
-                float &f = s_fold[c * NP + tid];
-                f = P ? f + v : v;
-            }
-#pragma unroll
-            for (int c = 0; c < 16; ++c) {
-                const float v = __uint_as_float(r1[c]) * is;
-                float &f = s_fold[(16 + c) * NP + tid];
-                f = P ? f + v : v;
             }
         };
 
-        form_coef();
+        // A entries: lane = 4 ylo + jp forms Ey of row y = 8 yq + ylo for visibilities 2 jp and 2 jp + 1
+        // of a group and multiplies the four polarisations with it (16 x 256-bit fragments)
+        const int jp = lane & 3;
+        const float Yv = (float)(8 * yq + (lane >> 2) - SL / 2);
+        const float ty = yq < NQ ? g.sep[SL + 8 * yq + (lane >> 2)] : 0.0f;
+        const f2_t Y2 = f2_pack(Yv, Yv), ty2 = f2_pack(ty, ty);
+        auto a_unit = [&](const float *cb, const float *vb, int pair, uint32_t (&e)[16]) {
+            const ulonglong2 cf = *(const ulonglong2 *)(cb + 4 * (pair + jp));
+            float p0, p1, sn0, cs0, sn1, cs1;
+            f2_unpack(f2_fma(cf.y, ty2, f2_mul(cf.x, Y2)), p0, p1);
+            __sincosf(p0, &sn0, &cs0);
+            __sincosf(p1, &sn1, &cs1);
+            const f2_t c2 = f2_pack(cs0, cs1), s2 = f2_pack(sn0, sn1), n2 = f2_mul(s2, f2_bcast(-1.0f));
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const ulonglong2 v = *(const ulonglong2 *)(vb + 2 * VB * q + 4 * (pair + jp));
+                f2_t hr, lr, hi, li;
+                f2_split(f2_fma(v.y, n2, f2_mul(v.x, c2)), magic_a, hr, lr);
+                f2_split(f2_fma(v.y, c2, f2_mul(v.x, s2)), magic_a, hi, li);
+                const int k = 8 * (q >> 1) + 2 * (q & 1);
+                pack_pairs(hr, hi, e[k], e[k + 1]);
+                pack_pairs(lr, li, e[k + 4], e[k + 5]);
+            }
+        };
+        // B entries of 8 pixel columns from 8 xblk for one group: lane = 8 jl + (x % 8), visibilities
+        // 2 jl and 2 jl + 1, which sit in adjacent K slots of each row: one 8-byte store per row (a
+        // warp's store covers 256 contiguous bytes).  beta = Ex_k(x) (m = 0: hi and lo) and c_k sigma
+        // Ex_k(x) (m = 1: hi), rows (m, re, x) = (Re beta, -Im beta) and (m, im, x) = (Im beta, Re beta)
+        const int jl = lane >> 3;
+        auto b_unit = [&](const float *ca, int pair, int xblk, f2_t X2, f2_t sx2, uint8_t *Bg) {
+            const ulonglong2 cf = *(const ulonglong2 *)(ca + 4 * (pair + jl));
+            float p0, p1, sn0, cs0, sn1, cs1;
+            f2_unpack(f2_fma(cf.y, sx2, f2_mul(cf.x, X2)), p0, p1);
+            __sincosf(p0, &sn0, &cs0);
+            __sincosf(p1, &sn1, &cs1);
+            const f2_t c2 = f2_pack(cs0, cs1), s2 = f2_pack(sn0, sn1), n2 = f2_mul(s2, f2_bcast(-1.0f));
+            const f2_t cz = f2_mul(cf.y, f2_pack(csig, csig)), zc = f2_mul(cz, c2), zs = f2_mul(cz, s2);
+            f2_t hc, lc, hs, ls, hn, ln;
+            f2_split(c2, magic_1, hc, lc);
+            f2_split(s2, magic_1, hs, ls);
+            f2_split(n2, magic_1, hn, ln);
+            uint32_t w[6][2];
+            pack_pairs(hc, hn, w[0][0], w[0][1]);
+            pack_pairs(hs, hc, w[1][0], w[1][1]);
+            pack_pairs(zc, f2_mul(cz, n2), w[2][0], w[2][1]);
+            pack_pairs(zs, zc, w[3][0], w[3][1]);
+            pack_pairs(lc, ln, w[4][0], w[4][1]);
+            pack_pairs(ls, lc, w[5][0], w[5][1]);
+            Bg += (uint32_t)xblk * kSBO + (uint32_t)(jl >> 1) * kLBO + (uint32_t)(lane & 7) * 16 + (uint32_t)(jl & 1) * 8;
+#pragma unroll
+            for (int q = 0; q < 6; ++q) *(uint2 *)(Bg + NQ * q * kSBO) = make_uint2(w[q][0], w[q][1]);
+        };
+        auto x_pair = [&](int xblk, f2_t &X2, f2_t &sx2) {
+            const int x = 8 * xblk + (lane & 7);
+            const float X = (float)(x - SL / 2), sx = g.sep[x];
+            X2 = f2_pack(X, X);
+            sx2 = f2_pack(sx, sx);
+        };
+        // this warp's x block: its own number at L = 32; at L = 24 and 16 the quarters without A
+        // rows take B blocks instead (16: quarters 2, 3 all of B; 24: quarter 3 the first group's)
+        const int xown = SL == 16 ? (yq & 1) : (SL == 24 && yq == 3 ? 0 : yq);
+        f2_t X2, sx2;
+        x_pair(xown, X2, sx2);
+
         store_batch(0);
         producers_sync();
         int next_fold = 0;
         for (int b = 0; b < n_batches; ++b) {
             const int bb = b & 1;
-            // this batch's power-of-two scale: largest |component| of V in [2^9, 2^10)
-            float m = 0.0f;
-#pragma unroll
-            for (int w = 0; w < NPW; ++w) m = fmaxf(m, s_red[bb][w]);
-            int e2 = 0;
-            if (m > 0.0f) frexpf(m, &e2);
-            const float scale = ldexpf(1.0f, 10 - e2);
-            if (bb) inv_sc1 = ldexpf(1.0f, e2 - 10);
-            else inv_sc0 = ldexpf(1.0f, e2 - 10);
             if (b + 1 < n_batches) load_batch(b + 1);
-            const float2 *cb = s_cb + bb * VB, *ca = s_ca + bb * VB;
-            const float2 *vb = s_vis + (size_t)bb * VB * 4;
-            const int nst = (min(GB, total_groups - b * GB) + SG - 1) / SG;
-            for (int si = 0; si < nst; ++si) {
-                const int st = b * (GB / SG) + si;
-                const int s = st % STAGES;
-                if (st >= STAGES) wait_or_fail(smem_u32(&s_empty[s]), (uint32_t)(((st / STAGES) - 1) & 1), failed);
-                // the MMAs of stage st - STAGES are done: when that was the last stage of period
-                // next_fold, read it out now (the next period's first MMA waits for it)
-                if (next_fold < n_batches - 1 && st - STAGES == (next_fold + 1) * (FOLD / SG) - 1) {
-                    fold(next_fold);
-                    ++next_fold;
-                }
-                // A entries of groups ga + 4 gg: scale V_kq Ey_k(y) for its 8 visibilities
+            const float *cb = s_cb + bb * VB * 2, *ca = s_ca + bb * VB * 2, *vb = s_vis + bb * VB * 8;
+            const int st_end = min((b + 1) * SPB, n_stages);
+            for (int st = b * SPB + set; st < st_end; st += 2) {
+                const int use = st >> 1, pair = (st - b * SPB) * (4 * SG);     // first visibility pair of the stage
+                const int ng = min(SG, total_groups - st * SG);
+                // B: the buffer's last reader was the set's stage before the previous one, waited for there
+                uint8_t *Bs = sB + (2 * set + (use & 1)) * B_STAGE;
+                if constexpr (SL == 32) {
 #pragma unroll
-                for (int gg = 0; gg < SG / 4; ++gg) {
-                    const int kb = 8 * (SG * si + ga + 4 * gg);
-                    float ec[2], es[2];
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const float2 cf = cb[kb + 2 * qa + h];
-                        float sn, cs;
-                        __sincosf(fmaf(cf.y, ty, cf.x * Yv), &sn, &cs);
-                        ec[h] = cs * scale;
-                        es[h] = sn * scale;
+                    for (int i = 0; i < SG; ++i)
+                        if (i < ng) b_unit(ca, pair + 4 * i, xown, X2, sx2, Bs + i * B_GROUP);
+                } else if constexpr (SL == 24) {
+                    if (yq < NQ) {
+                        if (ng > 1) b_unit(ca, pair + 4, xown, X2, sx2, Bs + B_GROUP);
+                    } else {
+#pragma unroll 1
+                        for (int xblk = 0; xblk < NQ; ++xblk) {
+                            x_pair(xblk, X2, sx2);
+                            b_unit(ca, pair, xblk, X2, sx2, Bs);
+                        }
                     }
-                    uint32_t e[16];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const int src = 8 * (j >> 1) + ylo;
-                        const float cs = __shfl_sync(0xffffffffu, (j & 1) ? ec[1] : ec[0], src);
-                        const float sn = __shfl_sync(0xffffffffu, (j & 1) ? es[1] : es[0], src);
-                        const float2 v = vb[(kb + j) * 4 + qa];
-                        split_e_m(fmaf(v.x, cs, -v.y * sn), fmaf(v.x, sn, v.y * cs), m1h, e[j], e[8 + j]);
-                        if (!row_ok) e[j] = e[8 + j] = 0u;
-                    }
-                    tmem_st16(lane_base + A_COL + 16u * SG * (uint32_t)s + 16u * (uint32_t)(ga + 4 * gg), e);
+                } else {
+                    if (yq >= NQ)
+                        for (int i = 0; i < ng; ++i) b_unit(ca, pair + 4 * i, xown, X2, sx2, Bs + i * B_GROUP);
                 }
-                // B entries: beta = Ex_k(x) (m = 0: hi and lo) and c_k sigma Ex_k(x) (m = 1: hi), rows
-                // (m, re, x) = (Re beta, -Im beta) and (m, im, x) = (Im beta, Re beta)
-                uint8_t *Bs = sB + s * B_STAGE;
+                // A: formed before, stored after the MMAs of the set's previous stage
+                if (yq < NQ) {
+                    const uint32_t ta = lane_base + A_COL + 16u * SG * (uint32_t)set;
 #pragma unroll
-                for (int gg = 0; gg < SG / 4; ++gg) {
-                    if (!x_ok) break;
-                    // visibilities j0 = 2 jl and j0 + 1 of group i = warp / 4 + 4 gg sit in adjacent K
-                    // slots of each row: one 8-byte store per row
-                    const int i = (warp >> 2) + 4 * gg, j0 = 2 * jl;
-                    uint32_t w[6][2];
-#pragma unroll
-                    for (int t = 0; t < 2; ++t) {
-                        const float2 cf = ca[8 * (SG * si + i) + j0 + t];
-                        float sn, cs;
-                        __sincosf(fmaf(cf.y, sx, cf.x * Xv), &sn, &cs);
-                        // the im row (sn, cs) is the re row (cs, -sn) with its halves swapped and the
-                        // new low half negated: exact, as FP16 rounding is symmetric
-                        uint32_t hr, lr;
-                        split_e_m(cs, -sn, m1h, hr, lr);
-                        const float cz = cf.y * csig;
-                        const uint32_t h1r = pack_f16x2(cz * cs, -cz * sn);
-                        w[0][t] = hr;
-                        w[1][t] = __byte_perm(hr, 0u, 0x1032u) ^ 0x8000u;
-                        w[2][t] = h1r;
-                        w[3][t] = __byte_perm(h1r, 0u, 0x1032u) ^ 0x8000u;
-                        w[4][t] = lr;
-                        w[5][t] = __byte_perm(lr, 0u, 0x1032u) ^ 0x8000u;
+                    for (int i = 0; i < SG; ++i) {
+                        uint32_t e[16];
+                        if (i < ng) a_unit(cb, vb, pair + 4 * i, e);
+                        if (i == 0 && use > 0) {
+                            wait_or_fail(smem_u32(&s_empty[set]), (uint32_t)((use - 1) & 1), failed);
+                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        }
+                        if (i < ng) {
+                            tmem_st_16x256b(ta + 16u * i, e);
+                            tmem_st_16x256b(ta + 16u * i + (16u << 16), e + 8);
+                        }
                     }
-                    uint8_t *Bg = Bs + i * B_GROUP + (uint32_t)(xb >> 3) * kSBO + (uint32_t)(jl >> 1) * kLBO +
-                                  (uint32_t)(xb & 7) * 16 + (uint32_t)(jl & 1) * 8;
-                    // row blocks of L (L / 8 kSBO): m = 0 re, m = 0 im, m = 1 re, m = 1 im, then the lo
-                    // parts of m = 0 re and im (rows 4 L + x, 5 L + x)
-#pragma unroll
-                    for (int q = 0; q < 6; ++q) *(uint2 *)(Bg + (SL / 8) * q * kSBO) = make_uint2(w[q][0], w[q][1]);
+                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                } else if (use > 0) {
+                    wait_or_fail(smem_u32(&s_empty[set]), (uint32_t)((use - 1) & 1), failed);
                 }
-                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&s_full[s]));
+                if (lane == 0) mbar_arrive(smem_u32(&s_full[set]));
+                // the set's first stage of a period is on its way: read out the period before
+                if (next_fold < st / SPP) {
+                    fold(next_fold);
+                    ++next_fold;
+                }
             }
             if (b + 1 < n_batches) {
-                form_coef();
                 store_batch(bb ^ 1);
                 producers_sync();
             }
         }
-        // the epilogue's global reads first: taper, and r(x, y) of this thread's x range
-        load_taper();
-        const int x0 = XS * sl;                     // this thread's x range in the epilogue
-        float rr_pre[XS];
-#pragma unroll
-        for (int xi = 0; xi < XS; ++xi) rr_pre[xi] = g.sep[2 * SL + yrow * SL + x0 + xi];
-        while (next_fold < n_batches) {
+        while (next_fold < n_periods) {
             fold(next_fold);
             ++next_fold;
         }
+        if (n_periods == 0)
+            for (int i = tid; i < 4 * SL * FFT_P; i += NP) s_img[i] = make_float2(0.f, 0.f);
         if (failed && lane == 0) atomicExch(&g_sep_error, 1);
-        producers_sync();      // every producer is past the stage and batch buffers and has folded
-        if (!failed && row_ok) {
-            // I = S0 + i r S1 / sigma into the polarisation planes.  Column C of the m = 0 block
-            // (re: C = x, im: C = L + x) was folded by the thread of slice C / 16 of this row,
-            // warp 4 (C / 16) + yq, as its entry C % 16.
-            const float rs = 1.0f / csig;
-#pragma unroll
-            for (int xi = 0; xi < XS; ++xi) {
-                const int x = x0 + xi, cre = x, cim = SL + x;
-                const int tre = (4 * (cre >> 4) + yq) * 32 + lane, tim = (4 * (cim >> 4) + yq) * 32 + lane;
-                float s0r = 0.f, s0i = 0.f, s1r = 0.f, s1i = 0.f;
-                if (n_batches) {
-                    s0r = s_fold[(cre & 15) * NP + tre];
-                    s0i = s_fold[(cim & 15) * NP + tim];
-                    s1r = s_fold[(16 + (cre & 15)) * NP + tre];
-                    s1i = s_fold[(16 + (cim & 15)) * NP + tim];
-                }
-                const float rr = rr_pre[xi] * rs;
-                s_fft[(qa * SL + yrow) * FFT_P + x] = make_float2(fmaf(-rr, s1i, s0r), fmaf(rr, s1r, s0i));
-            }
-        }
     }
+    // the taper of this thread's epilogue pixels
+    float tw_pre[PIXT];
+#pragma unroll
+    for (int i = 0; i < PIXT; ++i) tw_pre[i] = !mma_warp && tid + i * NP < SPIX ? taper[tid + i * NP] : 0.0f;
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     if (!__syncthreads_or(failed)) {
         if (aterms) {
@@ -483,53 +514,61 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
             if (late) atomicExch(&g_sep_error, 1);
         }
         // image-domain kernel per pixel: taper * A_p^H I A_q (with the centring factor when FUSED)
+        if (!mma_warp) {
 #pragma unroll
-        for (int ip = 0; ip < NPIX; ++ip) {
-            const int pix = tid + ip * NT;
-            if (pix >= SPIX) break;
-            const int y = pix / SL, x = pix % SL;
-            M22 P;
+            for (int ip = 0; ip < PIXT; ++ip) {
+                const int pix = tid + ip * NP;
+                if (pix >= SPIX) break;
+                const int y = pix / SL, x = pix % SL;
+                M22 P;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) P.m[c] = s_fft[(c * SL + y) * FFT_P + x];
-            if (d.dws != 0.0f) {      // the sums used w_s: the rest of the w offset, exp(i 2 pi (w_s - w0) n')
-                float sn, cs;
-                sincospif(d.dws * g.nprime[pix], &sn, &cs);     // (dws in half turns: exact reduction)
+                for (int c = 0; c < 4; ++c) P.m[c] = s_img[(c * SL + y) * FFT_P + x];
+                if (d.dws != 0.0f) {      // the sums used w_s: the rest of the w offset, exp(i 2 pi (w_s - w0) n')
+                    float sn, cs;
+                    sincospif(d.dws * g.nprime[pix], &sn, &cs);     // (dws in half turns: exact reduction)
 #pragma unroll
-                for (int c = 0; c < 4; ++c)
-                    P.m[c] = make_float2(P.m[c].x * cs - P.m[c].y * sn, P.m[c].x * sn + P.m[c].y * cs);
-            }
-            if (aterms) {
-                const float4 *at = (const float4 *)(smem + AT_OFF);
-                const M22 Ap = load_m22(at + 2 * pix);
-                const M22 Aq = load_m22(at + 2 * (SPIX + pix));
-                P = herm_mul_mul(Ap, P, Aq);
-            }
-            if (FUSED) {
-                const float tw = ((x + y) & 1) ? -tw_pre[ip] : tw_pre[ip];
+                    for (int c = 0; c < 4; ++c)
+                        P.m[c] = make_float2(P.m[c].x * cs - P.m[c].y * sn, P.m[c].x * sn + P.m[c].y * cs);
+                }
+                if (aterms) {
+                    const float4 *at = (const float4 *)(smem + AT_OFF);
+                    const M22 Ap = load_m22(at + 2 * pix);
+                    const M22 Aq = load_m22(at + 2 * (SPIX + pix));
+                    P = herm_mul_mul(Ap, P, Aq);
+                }
+                if (FUSED) {
+                    const float tw = ((x + y) & 1) ? -tw_pre[ip] : tw_pre[ip];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) s_fft[(c * SL + y) * FFT_P + x] = make_float2(tw * P.m[c].x, tw * P.m[c].y);
-            } else {
-                const float tw = tw_pre[ip];
-                o[2 * pix] = make_float4(tw * P.m[0].x, tw * P.m[0].y, tw * P.m[1].x, tw * P.m[1].y);
-                o[2 * pix + 1] = make_float4(tw * P.m[2].x, tw * P.m[2].y, tw * P.m[3].x, tw * P.m[3].y);
+                    for (int c = 0; c < 4; ++c)
+                        s_img[(c * SL + y) * FFT_P + x] = make_float2(tw * P.m[c].x, tw * P.m[c].y);
+                } else {
+                    const float tw = tw_pre[ip];
+                    o[2 * pix] = make_float4(tw * P.m[0].x, tw * P.m[0].y, tw * P.m[1].x, tw * P.m[1].y);
+                    o[2 * pix + 1] = make_float4(tw * P.m[2].x, tw * P.m[2].y, tw * P.m[3].x, tw * P.m[3].y);
+                }
             }
         }
         if (FUSED) {
             __syncthreads();
             if constexpr (SL == 32)
-                fft2_planar_pairs32<-1>(s_fft, tid);
+                fft2_planar_pairs32<-1>(s_img, tid);
             else
-                fft2_planar<SL, -1>(s_fft, tid, NT);
+                fft2_planar<SL, -1>(s_img, tid, NT);
             const float inv = 1.0f / (float)SPIX;
             float4 *dst = o + (size_t)d.layer * g.N * g.N * 2;
-            for (int pix = tid; pix < SPIX; pix += NT) {
-                const int i = pix / SL, j = pix % SL;
-                const float sg = ((i + j) & 1) ? -inv : inv;
-                const float2 p0 = s_fft[(0 * SL + i) * FFT_P + j], p1 = s_fft[(1 * SL + i) * FFT_P + j];
-                const float2 p2 = s_fft[(2 * SL + i) * FFT_P + j], p3 = s_fft[(3 * SL + i) * FFT_P + j];
-                const size_t gp = (size_t)(d.r0 + i) * g.N + (d.q0 + j);
-                red_add_f4(dst + 2 * gp, make_float4(sg * p0.x, sg * p0.y, sg * p1.x, sg * p1.y));
-                red_add_f4(dst + 2 * gp + 1, make_float4(sg * p2.x, sg * p2.y, sg * p3.x, sg * p3.y));
+            if (!mma_warp) {
+#pragma unroll
+                for (int ip = 0; ip < PIXT; ++ip) {
+                    const int pix = tid + ip * NP;
+                    if (pix >= SPIX) break;
+                    const int i = pix / SL, j = pix % SL;
+                    const float sg = ((i + j) & 1) ? -inv : inv;
+                    const float2 p0 = s_img[(0 * SL + i) * FFT_P + j], p1 = s_img[(1 * SL + i) * FFT_P + j];
+                    const float2 p2 = s_img[(2 * SL + i) * FFT_P + j], p3 = s_img[(3 * SL + i) * FFT_P + j];
+                    const size_t gp = (size_t)(d.r0 + i) * g.N + (d.q0 + j);
+                    red_add_f4(dst + 2 * gp, make_float4(sg * p0.x, sg * p0.y, sg * p1.x, sg * p1.y));
+                    red_add_f4(dst + 2 * gp + 1, make_float4(sg * p2.x, sg * p2.y, sg * p3.x, sg * p3.y));
+                }
             }
         }
     }
@@ -538,12 +577,13 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
         bool late = false;
         wait_or_fail(smem_u32(&s_atbar), 0u, late);
     }
-    if (mma_warp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "n"(512));
+    if (mma_warp)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "n"(TMEM_COLS));
 }
 
 // one CTA per subgrid of one plan (plan index idx[b] or first + b): subgrid images
 template <int L>
-__global__ void __launch_bounds__(NT, 1)
+__global__ void __launch_bounds__(NT, CTAS)
 gridder_sep_kernel(Geometry g, const int32_t *__restrict__ idx, int64_t first, const float4 *__restrict__ vis,
                    const uint8_t *__restrict__ flags, const float4 *__restrict__ aterms,
                    const float *__restrict__ taper, float4 *__restrict__ out) {
@@ -553,7 +593,7 @@ gridder_sep_kernel(Geometry g, const int32_t *__restrict__ idx, int64_t first, c
 
 // fused: one CTA per subgrid, transformed and added into the grid
 template <int L>
-__global__ void __launch_bounds__(NT, 1)
+__global__ void __launch_bounds__(NT, CTAS)
 gridder_sep_fused_kernel(Geometry g, const int32_t *__restrict__ idx, int64_t first, const float4 *__restrict__ vis,
                          const uint8_t *__restrict__ flags, const float4 *__restrict__ aterms,
                          const float *__restrict__ taper, float4 *__restrict__ grid) {

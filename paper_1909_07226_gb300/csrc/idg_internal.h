@@ -51,6 +51,7 @@ struct Geometry {
     // max |r| smallest), r the remainder; sep = [s[L] | t[L] | r[L][L]] (FP64
     // differences rounded to FP32)
     const float *sep;
+    float sep_s[32], sep_t[32];    // s and t again, as kernel parameters (constant operands); L <= 32
     // 1: the launch's subgrids meet the bound max |c_k| max |r| of the first-order w
     // remainder (the plan's own value: every subgrid does; the composite calls set it
     // per launch for the separable part of a plan)
@@ -101,6 +102,7 @@ struct idg_plan {
     float *d_nprime = nullptr;             // [L][L] n', then the separable tables [2 L + L^2]
     double sep_theta = 0.0;                // max |c_k| max |r(x, y)|: phase of the separable remainder
     int sep_j0 = 0;                        // reference row and column of the separable split
+    float sep_s[32] = {}, sep_t[32] = {};  // its s(x) and t(y), L <= 32 (host copy)
     // per subgrid (plan order): the separable kernels' w offset w_s (wavelengths), and
     // 1 where the remainder phase with it meets the bound (the separable kernels take it)
     std::vector<double> w_sep;

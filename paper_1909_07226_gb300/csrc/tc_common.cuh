@@ -128,6 +128,24 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[16]) {
                  :: "memory");
 }
 
+// 4 columns, as above
+__device__ __forceinline__ void tmem_ld_nowait(uint32_t taddr, uint32_t (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[4]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]) :: "memory");
+}
+
+// 16 tensor-memory lanes (a half of the warp's 32) x 16 columns as two 8 x 8-column fragments:
+// thread t holds lanes t / 4 (v[0], v[1]) and t / 4 + 8 (v[2], v[3]) of columns 2 (t % 4) and
+// + 1, v[4 ..] the same of columns 8 .. 15
+__device__ __forceinline__ void tmem_st_16x256b(uint32_t taddr, const uint32_t *v) {
+    asm volatile("tcgen05.st.sync.aligned.16x256b.x2.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                 :: "r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+}
+
 // 8 or 4 columns of the warp's 32 lanes (complete after tcgen05.wait::st)
 __device__ __forceinline__ void tmem_st(uint32_t taddr, const uint32_t (&v)[8]) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
@@ -168,6 +186,15 @@ __device__ __forceinline__ uint32_t pack_f16x2(float x, float y) {
     uint32_t r;
     asm("cvt.rn.f16x2.f32 %0, %2, %1;" : "=r"(r) : "f"(x), "f"(y));
     return r;
+}
+
+// FP16 pairs (x0, y0) and (x1, y1) of packed (x0, x1) and (y0, y1)
+__device__ __forceinline__ void pack_pairs(unsigned long long x, unsigned long long y, uint32_t &w0, uint32_t &w1) {
+    float x0, x1, y0, y1;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x0), "=f"(x1) : "l"(x));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(y0), "=f"(y1) : "l"(y));
+    w0 = pack_f16x2(x0, y0);
+    w1 = pack_f16x2(x1, y1);
 }
 
 // FP16 hi/lo parts of (x, y): hi = fp16 rounded, lo = fp16(v - hi) with v - hi formed
