@@ -77,9 +77,11 @@ struct SepD {
     // B (fixed per subgrid), each [KT][part][PN rows][16 K]: Q0 hi, Q0 lo, Q1 hi
     static constexpr int TB = 8 * L * 32;           // one K step: 8 L rows x 32 bytes
     static constexpr int B0L = KT * TB, B1H = 2 * KT * TB, B_BYTES = 3 * KT * TB;
-    // prologue scratch over B: the subgrid's grid rows, then the transform planes
-    static constexpr int FFT_P = L + 1, FFT_OFF = SPIX * 32, FFT_BYTES = 4 * L * FFT_P * 8;
-    static constexpr int PART_OFF = B_BYTES > FFT_OFF + FFT_BYTES ? B_BYTES : FFT_OFF + FFT_BYTES;
+    // prologue scratch over B: the subgrid's grid rows, then (with 4 float2 of row padding) its image,
+    // pixel by pixel; behind them the transform planes
+    static constexpr int FFT_P = PolPlanes<L>::P, FFT_S = PolPlanes<L>::STRIDE;
+    static constexpr int PIX_P = 4 * L + 4, FFT_OFF = L * PIX_P * 8, FFT_END = FFT_OFF + 4 * FFT_S * 8;
+    static constexpr int PART_OFF = B_BYTES > FFT_END ? B_BYTES : FFT_END;
     static constexpr int SMEM = PART_OFF + 2 * 2 * TV * 16;      // [2 tiles][2 pol pairs][TV] float4 (y halves meet)
     // tensor memory: accumulator, then A hi, lo and m = 1, one column per x
     static constexpr uint32_t A_COL = PN;
@@ -164,9 +166,8 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
                                                    const float4 *__restrict__ aterms, const float *__restrict__ taper,
                                                    float4 *__restrict__ vis_out) {
     using C = SepD<L>;
-    constexpr int SL = C::SL, SPIX = C::SPIX, KT = C::KT, FFT_P = C::FFT_P, H = C::H, YB = C::YB, QH = C::QH;
+    constexpr int SL = C::SL, SPIX = C::SPIX, KT = C::KT, H = C::H, YB = C::YB, QH = C::QH;
     extern __shared__ __align__(1024) uint8_t smem[];
-    float2 *s_fft = (float2 *)(smem + C::FFT_OFF);       // [4][L][L + 1] during the prologue
     float4 *s_part = (float4 *)(smem + C::PART_OFF);
     __shared__ uint32_t s_tmem;
     __shared__ __align__(8) uint64_t s_afull, s_dfull, s_dempty, s_drain, s_gbar;
@@ -236,21 +237,20 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
         bool late = false;
         wait_or_fail(smem_u32(&s_gbar), 0u, late);
         if (late) atomicExch(&g_sepd_error, 1);
-        const float4 *rows = (const float4 *)smem;
-        for (int pix = tid; pix < SPIX; pix += NT) {
-            const int i = pix / SL, j = pix % SL;
-            const float sg = ((i + j) & 1) ? -1.0f : 1.0f;
-            const float4 a = rows[2 * pix], b = rows[2 * pix + 1];
-            s_fft[(0 * SL + i) * FFT_P + j] = make_float2(sg * a.x, sg * a.y);
-            s_fft[(1 * SL + i) * FFT_P + j] = make_float2(sg * a.z, sg * a.w);
-            s_fft[(2 * SL + i) * FFT_P + j] = make_float2(sg * b.x, sg * b.y);
-            s_fft[(3 * SL + i) * FFT_P + j] = make_float2(sg * b.z, sg * b.w);
+        // one thread per line and polarisation: columns from the grid rows, then rows into the image
+        const int pol = tid & 3, ln = tid >> 2;
+        const float2 *src_col = (const float2 *)smem + 4 * ln + pol;
+        float2 *plane = (float2 *)(smem + C::FFT_OFF) + pol * C::FFT_S;
+        if (tid < 4 * SL)
+            fft_line<SL, +1>([&](int n) { return src_col[n * 4 * SL]; },
+                             [&](int k, float2 v) { plane[k * C::FFT_P + ln] = v; });
+        __syncthreads();
+        if (tid < 4 * SL) {
+            const float2 *row = plane + ln * C::FFT_P;
+            float2 *dst = (float2 *)smem + ln * C::PIX_P + pol;
+            fft_line<SL, +1>([&](int n) { return row[n]; }, [&](int k, float2 v) { dst[4 * k] = v; });
         }
         __syncthreads();
-        if constexpr (SL == 32)
-            fft2_planar_pairs32<+1>(s_fft, tid);
-        else
-            fft2_planar<SL, +1>(s_fft, tid, NT);
     }
     M22 P[C::TPW];
     if (warp < NWW) {
@@ -260,16 +260,7 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
             const int tile = warp + NWW * i;
             if (tile >= C::NTILE) break;
             const int y = 8 * (tile / (SL / 4)) + (lane >> 2), x = 4 * (tile % (SL / 4)) + (lane & 3), pix = y * SL + x;
-            if (FUSED) {      // (-1)^(x+y) / L^2 of the transform
-                const float sg = ((x + y) & 1) ? -1.0f / SPIX : 1.0f / SPIX;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float2 v = s_fft[(q * SL + y) * FFT_P + x];
-                    P[i].m[q] = make_float2(sg * v.x, sg * v.y);
-                }
-            } else {
-                P[i] = load_m22(src + 2 * pix);
-            }
+            P[i] = load_m22(FUSED ? (const float4 *)smem + y * (C::PIX_P / 2) + 2 * x : src + 2 * pix);
             if (d.dws != 0.0f) {      // the sums use w_s: the rest of the w offset, exp(-i 2 pi (w_s - w0) n')
                 float sn, cs;
                 sincospif(d.dws * g.nprime[pix], &sn, &cs);     // (dws in half turns: exact reduction)
@@ -283,7 +274,7 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
                 const M22 Aq = load_m22(base + 2 * (size_t)d.st_q * SPIX);
                 P[i] = mul_mul_herm(Ap, P[i], Aq);
             }
-            const float tw = taper[pix];
+            const float tw = FUSED ? taper[pix] * (1.0f / SPIX) : taper[pix];      // with the transform's L^-2
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 P[i].m[q] = make_float2(tw * P[i].m[q].x, tw * P[i].m[q].y);
@@ -345,10 +336,10 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
             const uint64_t db0 = smem_desc(smem_u32(smem));
             const uint32_t at = tmem + C::A_COL;
             for (int t = 0; t < n_tiles; ++t) {
-                wait_or_fail(smem_u32(&s_afull), (uint32_t)(t & 1), failed);
+                poll_or_fail(smem_u32(&s_afull), (uint32_t)(t & 1), failed);
                 for (int p = 0; p < C::PARTS; ++p) {
                     const int n = t * C::PARTS + p;
-                    if (n > 0) wait_or_fail(smem_u32(&s_dempty), (uint32_t)((n - 1) & 1), failed);
+                    if (n > 0) poll_or_fail(smem_u32(&s_dempty), (uint32_t)((n - 1) & 1), failed);
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint64_t dbp = db0 + (uint64_t)((p * C::PN * 32) >> 4);
 #pragma unroll

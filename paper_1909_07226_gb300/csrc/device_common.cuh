@@ -75,6 +75,11 @@ __device__ __forceinline__ void red_add_f4(float4 *p, float4 v) {
                  : "memory");
 }
 
+// the same for 8 bytes
+__device__ __forceinline__ void red_add_f2(float2 *p, float2 v) {
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" :: "l"(p), "f"(v.x), "f"(v.y) : "memory");
+}
+
 __device__ __forceinline__ size_t vis_index(const Geometry &g, const DevSubgrid &d, int k, int &t, int &c) {
     const int tt = k / d.nc;
     t = d.t0 + tt;

@@ -92,9 +92,9 @@ struct SepG {
     static constexpr int SL = L, SPIX = L * L, NQ = L / 8;   // NQ: 8-row (and 8-column) blocks
     static constexpr int B_GROUP = 6 * L * 32;   // B of one group: 6 L rows x 16 K FP16
     static constexpr int B_STAGE = SG * B_GROUP;
-    // the subgrid image (polarisation planes, row pitch L + 1): the folded sums, then transformed in place
-    static constexpr int FFT_P = L + 1, IMG_BYTES = 4 * L * FFT_P * 8;
-    static constexpr int B_OFF = IMG_BYTES;      // [2 sets][2 buffers][SG groups]
+    // the subgrid image (polarisation planes, row pitch L + 1): the folded sums, then transformed
+    static constexpr int FFT_P = PolPlanes<L>::P, FFT_S = PolPlanes<L>::STRIDE;
+    static constexpr int B_OFF = (4 * FFT_S * 8 + 127) / 128 * 128;      // [2 sets][2 buffers][SG groups]
     // staged batches, [2] each, visibility pairs: (b0, b1, c0, c1), (a0, a1, c0, c1) and per
     // polarisation (re0, re1, im0, im1)
     static constexpr int CB_OFF = B_OFF + 4 * B_STAGE, CA_OFF = CB_OFF + 2 * VB * 8;
@@ -128,10 +128,10 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
                                                  float4 *__restrict__ o) {
     using C = SepG<L>;
     constexpr int SL = C::SL, SPIX = C::SPIX, NQ = C::NQ, B_GROUP = C::B_GROUP, B_STAGE = C::B_STAGE;
-    constexpr int FFT_P = C::FFT_P, AT_OFF = C::AT_OFF, XS = C::XS, PIXT = C::PIXT;
+    constexpr int FFT_P = C::FFT_P, FFT_S = C::FFT_S, AT_OFF = C::AT_OFF, XS = C::XS, PIXT = C::PIXT;
     constexpr uint32_t AT_BYTES = C::AT_BYTES, A_COL = C::A_COL;
     extern __shared__ __align__(1024) uint8_t smem[];
-    float2 *s_img = (float2 *)smem;                 // [4][L][L + 1]
+    float2 *s_img = (float2 *)smem;                 // 4 planes [L][L + 1]
     uint8_t *sB = smem + C::B_OFF;
     float *s_cb = (float *)(smem + C::CB_OFF), *s_ca = (float *)(smem + C::CA_OFF);
     float *s_vis = (float *)(smem + C::VIS_OFF);
@@ -240,7 +240,7 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
                 if (first && st > 0) {         // the producers have read the previous period
                     wait_or_fail(smem_u32(&s_folded), (uint32_t)(((st / SPP) - 1) & 1), failed);
                 }
-                wait_or_fail(smem_u32(&s_full[s]), (uint32_t)(use & 1), failed);
+                poll_or_fail(smem_u32(&s_full[s]), (uint32_t)(use & 1), failed);
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const int ng = min(SG, total_groups - st * SG);
                 const uint64_t dbs = db0 + (uint64_t)(((2 * s + (use & 1)) * B_STAGE) >> 4);
@@ -325,7 +325,7 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
             constexpr int XC = C::XC;
             if (yq < NQ) {
                 const int y = 8 * yq + (lane & 7);
-                float2 *img = s_img + ((lane >> 3) * SL + y) * FFT_P + set * XS;
+                float2 *img = s_img + (lane >> 3) * FFT_S + y * FFT_P + set * XS;
                 const float *rp = g.sep + 2 * SL + y * SL + set * XS;
 #pragma unroll
                 for (int x0 = 0; x0 < XS; x0 += XC) {
@@ -499,7 +499,7 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
             ++next_fold;
         }
         if (n_periods == 0)
-            for (int i = tid; i < 4 * SL * FFT_P; i += NP) s_img[i] = make_float2(0.f, 0.f);
+            for (int i = tid; i < 4 * FFT_S; i += NP) s_img[i] = make_float2(0.f, 0.f);
         if (failed && lane == 0) atomicExch(&g_sep_error, 1);
     }
     // the taper of this thread's epilogue pixels
@@ -522,7 +522,7 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
                 const int y = pix / SL, x = pix % SL;
                 M22 P;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) P.m[c] = s_img[(c * SL + y) * FFT_P + x];
+                for (int c = 0; c < 4; ++c) P.m[c] = s_img[c * FFT_S + y * FFT_P + x];
                 if (d.dws != 0.0f) {      // the sums used w_s: the rest of the w offset, exp(i 2 pi (w_s - w0) n')
                     float sn, cs;
                     sincospif(d.dws * g.nprime[pix], &sn, &cs);     // (dws in half turns: exact reduction)
@@ -537,10 +537,10 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
                     P = herm_mul_mul(Ap, P, Aq);
                 }
                 if (FUSED) {
-                    const float tw = ((x + y) & 1) ? -tw_pre[ip] : tw_pre[ip];
+                    const float tw = tw_pre[ip] * (1.0f / SPIX);      // with the transform's L^-2
 #pragma unroll
                     for (int c = 0; c < 4; ++c)
-                        s_img[(c * SL + y) * FFT_P + x] = make_float2(tw * P.m[c].x, tw * P.m[c].y);
+                        s_img[c * FFT_S + y * FFT_P + x] = make_float2(tw * P.m[c].x, tw * P.m[c].y);
                 } else {
                     const float tw = tw_pre[ip];
                     o[2 * pix] = make_float4(tw * P.m[0].x, tw * P.m[0].y, tw * P.m[1].x, tw * P.m[1].y);
@@ -550,25 +550,21 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
         }
         if (FUSED) {
             __syncthreads();
-            if constexpr (SL == 32)
-                fft2_planar_pairs32<-1>(s_img, tid);
-            else
-                fft2_planar<SL, -1>(s_img, tid, NT);
-            const float inv = 1.0f / (float)SPIX;
-            float4 *dst = o + (size_t)d.layer * g.N * g.N * 2;
-            if (!mma_warp) {
-#pragma unroll
-                for (int ip = 0; ip < PIXT; ++ip) {
-                    const int pix = tid + ip * NP;
-                    if (pix >= SPIX) break;
-                    const int i = pix / SL, j = pix % SL;
-                    const float sg = ((i + j) & 1) ? -inv : inv;
-                    const float2 p0 = s_img[(0 * SL + i) * FFT_P + j], p1 = s_img[(1 * SL + i) * FFT_P + j];
-                    const float2 p2 = s_img[(2 * SL + i) * FFT_P + j], p3 = s_img[(3 * SL + i) * FFT_P + j];
-                    const size_t gp = (size_t)(d.r0 + i) * g.N + (d.q0 + j);
-                    red_add_f4(dst + 2 * gp, make_float4(sg * p0.x, sg * p0.y, sg * p1.x, sg * p1.y));
-                    red_add_f4(dst + 2 * gp + 1, make_float4(sg * p2.x, sg * p2.y, sg * p3.x, sg * p3.y));
-                }
+            // one thread per line and polarisation: rows in place, then columns, which leave with
+            // 8-byte reductions (the 8 columns x 4 polarisations of a warp are 256 contiguous bytes
+            // of a grid row)
+            const int pol = tid & 3, ln = tid >> 2;
+            float2 *plane = s_img + pol * FFT_S;
+            if (tid < 4 * SL) {
+                float2 *row = plane + ln * FFT_P;
+                fft_line<SL, -1>([&](int n) { return row[n]; }, [&](int k, float2 v) { row[k] = v; });
+            }
+            __syncthreads();
+            if (tid < 4 * SL) {
+                float2 *dst = (float2 *)o + ((((size_t)d.layer * g.N + d.r0) * g.N + d.q0 + ln) * 4 + pol);
+                const size_t pitch = (size_t)g.N * 4;
+                fft_line<SL, -1>([&](int n) { return plane[n * FFT_P + ln]; },
+                                 [&](int k, float2 v) { red_add_f2(dst + k * pitch, v); });
             }
         }
     }

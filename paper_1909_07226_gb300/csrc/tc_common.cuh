@@ -84,6 +84,21 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     return false;
 }
 
+// the same wait without suspending the thread, for the one thread that issues the MMAs (it
+// starts them a little sooner; worker warps that poll cost the others issue slots)
+__device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity) {
+    for (long it = 0; it < kSpin; ++it) {
+        uint32_t ok;
+        asm volatile("{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+                     " selp.u32 %0, 1, 0, p;\n}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        if (ok) return true;
+    }
+    return false;
+}
+__device__ __forceinline__ void poll_or_fail(uint32_t bar, uint32_t parity, bool &failed) {
+    if (!failed && !mbar_poll(bar, parity)) failed = true;
+}
+
 // a bounded wait that is skipped once this thread has seen a failure, so that
 // control flow stays uniform and the kernel ends
 __device__ __forceinline__ void wait_or_fail(uint32_t bar, uint32_t parity, bool &failed) {
