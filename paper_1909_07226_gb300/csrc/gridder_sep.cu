@@ -436,53 +436,57 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
             if (b + 1 < n_batches) load_batch(b + 1);
             const float *cb = s_cb + bb * VB * 2, *ca = s_ca + bb * VB * 2, *vb = s_vis + bb * VB * 8;
             const int st_end = min((b + 1) * SPB, n_stages);
-            for (int st = b * SPB + set; st < st_end; st += 2) {
-                const int use = st >> 1, pair = (st - b * SPB) * (4 * SG);     // first visibility pair of the stage
-                const int ng = min(SG, total_groups - st * SG);
-                // B: the buffer's last reader was the set's stage before the previous one, waited for there
-                uint8_t *Bs = sB + (2 * set + (use & 1)) * B_STAGE;
-                if constexpr (SL == 32) {
-#pragma unroll
-                    for (int i = 0; i < SG; ++i)
-                        if (i < ng) b_unit(ca, pair + 4 * i, xown, X2, sx2, Bs + i * B_GROUP);
-                } else if constexpr (SL == 24) {
+            // B of the stage's first (half 0) or second group (half 1); at L = 24 quarter 3 does the first
+            // group's three blocks, 0 and 1 in half 0
+            auto b_half = [&](int st, int half) {
+                const int pair = (st - b * SPB) * (4 * SG);      // first visibility pair of the stage
+                uint8_t *Bs = sB + (2 * set + ((st >> 1) & 1)) * B_STAGE;
+                if (half && st * SG + 1 >= total_groups && !(SL == 24 && yq == 3)) return;
+                if constexpr (SL == 24) {
                     if (yq < NQ) {
-                        if (ng > 1) b_unit(ca, pair + 4, xown, X2, sx2, Bs + B_GROUP);
+                        if (half) b_unit(ca, pair + 4, yq, X2, sx2, Bs + B_GROUP);
                     } else {
-#pragma unroll 1
-                        for (int xblk = 0; xblk < NQ; ++xblk) {
+                        for (int xblk = 2 * half; xblk < 2 + half; ++xblk) {
                             x_pair(xblk, X2, sx2);
                             b_unit(ca, pair, xblk, X2, sx2, Bs);
                         }
                     }
                 } else {
-                    if (yq >= NQ)
-                        for (int i = 0; i < ng; ++i) b_unit(ca, pair + 4 * i, xown, X2, sx2, Bs + i * B_GROUP);
+                    if (SL == 32 || yq >= NQ) b_unit(ca, pair + 4 * half, xown, X2, sx2, Bs + half * B_GROUP);
                 }
-                // A: formed before, stored after the MMAs of the set's previous stage
+            };
+            const int st0 = b * SPB + set;
+            if (st0 < st_end) b_half(st0, 0);
+            for (int st = st0; st < st_end; st += 2) {
+                const int use = st >> 1, pair = (st - b * SPB) * (4 * SG);
+                const bool two = st * SG + 1 < total_groups;
                 if (yq < NQ) {
                     const uint32_t ta = lane_base + A_COL + 16u * SG * (uint32_t)set;
-#pragma unroll
-                    for (int i = 0; i < SG; ++i) {
-                        uint32_t e[16];
-                        if (i < ng) a_unit(cb, vb, pair + 4 * i, e);
-                        if (i == 0 && use > 0) {
-                            wait_or_fail(smem_u32(&s_empty[set]), (uint32_t)((use - 1) & 1), failed);
-                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        }
-                        if (i < ng) {
-                            tmem_st_16x256b(ta + 16u * i, e);
-                            tmem_st_16x256b(ta + 16u * i + (16u << 16), e + 8);
-                        }
+                    uint32_t e[16];
+                    a_unit(cb, vb, pair, e);
+                    if (use > 0) {       // the MMAs of the set's previous stage are done with A
+                        wait_or_fail(smem_u32(&s_empty[set]), (uint32_t)((use - 1) & 1), failed);
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     }
-                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                    tmem_st_16x256b(ta, e);
+                    tmem_st_16x256b(ta + (16u << 16), e + 8);
+                    if (two) {
+                        a_unit(cb, vb, pair + 4, e);
+                        tmem_st_16x256b(ta + 16u, e);
+                        tmem_st_16x256b(ta + 16u + (16u << 16), e + 8);
+                    }
                 } else if (use > 0) {
                     wait_or_fail(smem_u32(&s_empty[set]), (uint32_t)((use - 1) & 1), failed);
                 }
+                // the second half of B while the tensor-memory stores land; the next stage's first half
+                // follows the arrival (its buffer's last reader was the stage waited for above)
+                b_half(st, 1);
+                if (yq < NQ) asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&s_full[set]));
+                if (st + 2 < st_end) b_half(st + 2, 0);
                 // the set's first stage of a period is on its way: read out the period before
                 if (next_fold < st / SPP) {
                     fold(next_fold);
