@@ -437,11 +437,9 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
             const float *cb = s_cb + bb * VB * 2, *ca = s_ca + bb * VB * 2, *vb = s_vis + bb * VB * 8;
             const int st_end = min((b + 1) * SPB, n_stages);
             // B of the stage's first (half 0) or second group (half 1); at L = 24 quarter 3 does the first
-            // group's three blocks, 0 and 1 in half 0
-            auto b_half = [&](int st, int half) {
-                const int pair = (st - b * SPB) * (4 * SG);      // first visibility pair of the stage
-                uint8_t *Bs = sB + (2 * set + ((st >> 1) & 1)) * B_STAGE;
-                if (half && st * SG + 1 >= total_groups && !(SL == 24 && yq == 3)) return;
+            // group's three blocks, 0 and 1 in half 0.  (A group past the last is staged zeros, which no
+            // MMA reads.)
+            auto b_half = [&](int pair, uint8_t *Bs, int half) {
                 if constexpr (SL == 24) {
                     if (yq < NQ) {
                         if (half) b_unit(ca, pair + 4, yq, X2, sx2, Bs + B_GROUP);
@@ -455,38 +453,33 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
                     if (SL == 32 || yq >= NQ) b_unit(ca, pair + 4 * half, xown, X2, sx2, Bs + half * B_GROUP);
                 }
             };
-            const int st0 = b * SPB + set;
-            if (st0 < st_end) b_half(st0, 0);
-            for (int st = st0; st < st_end; st += 2) {
-                const int use = st >> 1, pair = (st - b * SPB) * (4 * SG);
-                const bool two = st * SG + 1 < total_groups;
+            int pair = set * (4 * SG);      // first visibility pair of the stage
+            for (int st = b * SPB + set; st < st_end; st += 2, pair += 8 * SG) {
+                const int use = st >> 1;
+                const uint32_t ta = lane_base + A_COL + 16u * SG * (uint32_t)set;
+                uint8_t *Bs = sB + (2 * set + (use & 1)) * B_STAGE;
+                // A and B of a group side by side, so that their chains (phase, sine and cosine, split)
+                // overlap.  The B buffer's last reader was the stage before the one waited for here
+                uint32_t e[16];
+                if (yq < NQ) a_unit(cb, vb, pair, e);
+                b_half(pair, Bs, 0);
+                if (use > 0) {       // the MMAs of the set's previous stage are done with A
+                    wait_or_fail(smem_u32(&s_empty[set]), (uint32_t)((use - 1) & 1), failed);
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                }
                 if (yq < NQ) {
-                    const uint32_t ta = lane_base + A_COL + 16u * SG * (uint32_t)set;
-                    uint32_t e[16];
-                    a_unit(cb, vb, pair, e);
-                    if (use > 0) {       // the MMAs of the set's previous stage are done with A
-                        wait_or_fail(smem_u32(&s_empty[set]), (uint32_t)((use - 1) & 1), failed);
-                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    }
                     tmem_st_16x256b(ta, e);
                     tmem_st_16x256b(ta + (16u << 16), e + 8);
-                    if (two) {
-                        a_unit(cb, vb, pair + 4, e);
-                        tmem_st_16x256b(ta + 16u, e);
-                        tmem_st_16x256b(ta + 16u + (16u << 16), e + 8);
-                    }
-                } else if (use > 0) {
-                    wait_or_fail(smem_u32(&s_empty[set]), (uint32_t)((use - 1) & 1), failed);
+                    a_unit(cb, vb, pair + 4, e);
+                    tmem_st_16x256b(ta + 16u, e);
+                    tmem_st_16x256b(ta + 16u + (16u << 16), e + 8);
                 }
-                // the second half of B while the tensor-memory stores land; the next stage's first half
-                // follows the arrival (its buffer's last reader was the stage waited for above)
-                b_half(st, 1);
+                b_half(pair, Bs, 1);
                 if (yq < NQ) asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&s_full[set]));
-                if (st + 2 < st_end) b_half(st + 2, 0);
                 // the set's first stage of a period is on its way: read out the period before
                 if (next_fold < st / SPP) {
                     fold(next_fold);
