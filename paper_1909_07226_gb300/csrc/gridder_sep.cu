@@ -75,7 +75,8 @@ using namespace tc;
 
 constexpr int NPW = 8;                         // producer warps: two sets of four
 constexpr int NP = NPW * 32;                   // producer threads
-constexpr int NT = NP + 32;                    // + the MMA warp
+constexpr int MMA_WARP = NPW, LOAD_WARP = NPW + 1;
+constexpr int NT = NP + 64;
 constexpr int CTAS = 2;                        // per SM
 constexpr int VB = NP;                         // visibilities per staged batch (one per producer)
 constexpr int SG = 2;                          // groups of 8 visibilities per stage
@@ -136,76 +137,122 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
     float *s_cb = (float *)(smem + C::CB_OFF), *s_ca = (float *)(smem + C::CA_OFF);
     float *s_vis = (float *)(smem + C::VIS_OFF);
     __shared__ uint32_t s_tmem;
-    __shared__ __align__(8) uint64_t s_full[2], s_empty[2], s_foldbar, s_folded, s_drain, s_atbar;
+    __shared__ __align__(8) uint64_t s_full[2], s_empty[2], s_foldbar, s_folded, s_drain, s_atbar,
+        s_staged, s_unstaged;
     __shared__ float s_red[NPW];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const bool mma_warp = warp == NPW;
+    const bool mma_warp = warp == MMA_WARP, producer = warp < NPW;
     const int kp = d.kp;
     const int total_groups = (kp + 7) / 8, n_stages = (total_groups + SG - 1) / SG;
     const int n_batches = (kp + VB - 1) / VB, n_periods = (n_stages + SPP - 1) / SPP;
 
-    // staging (producers): visibility tid of batch b, loaded into registers one batch ahead;
-    // the first batch's loads go out before the set-up below, so their latency overlaps it
-    float4 pa = make_float4(0.f, 0.f, 0.f, 0.f), pb = pa, puv = pa, pws = pa;
-    float2 pw = make_float2(0.f, 0.f);
-    bool pin = false, pflag = false;
+    // staging: one visibility's inputs in registers, then its phase coefficients and scaled
+    // values in shared memory.  The producers stage the first batch (its loads go out before
+    // the set-up below, so their latency overlaps it), a loader warp the others
+    struct Raw {
+        float4 a, b, uv, sc;
+        float2 w;
+        bool in, flag;
+    };
     const float4 *uvw2 = (const float4 *)g.uvw_f2;
     const float4 *sc2 = (const float4 *)g.scale_f2;
     const size_t bt0 = (size_t)d.bl * g.n_t + d.t0;
-    const int dt = VB / d.nc, dc = VB - dt * d.nc;     // a batch's step in timestep and channel
-    const int vt0 = tid / d.nc, vc0 = tid - vt0 * d.nc;
-    int vt = vt0, vc = vc0;
-    auto advance = [&](int &t, int &c) {
-        t += dt;
-        c += dc;
-        if (c >= d.nc) {
-            c -= d.nc;
-            ++t;
+    auto load = [&](Raw &r, bool in, int t, int c) {
+        r.in = in;
+        r.flag = false;
+        if (in) {
+            const size_t bt = bt0 + t;
+            const size_t vi = bt * g.n_chan + d.c0 + c;
+            r.uv = uvw2[2 * bt];
+            r.w = *(const float2 *)(uvw2 + 2 * bt + 1);
+            r.sc = sc2[d.c0 + c];
+            r.flag = flags && flags[vi];
+            r.a = vis[2 * vi];         // loaded whatever the flag: the load does not wait for it
+            r.b = vis[2 * vi + 1];
         }
     };
-    auto load_batch = [&](int b) {
-        pin = b * VB + tid < kp;
-        pflag = false;
-        if (pin) {
-            const size_t bt = bt0 + vt;
-            const int c = d.c0 + vc;
-            const size_t vi = bt * g.n_chan + c;
-            puv = uvw2[2 * bt];
-            pw = *(const float2 *)(uvw2 + 2 * bt + 1);
-            pws = sc2[c];
-            pflag = flags && flags[vi];
-            pa = vis[2 * vi];          // loaded whatever the flag: the load does not wait for it
-            pb = vis[2 * vi + 1];
+    // slot i of staging buffer bb: phase coefficients u (f/c) k_uv - u0 k_uv and so on (float
+    // pairs, error-free products and sums, rounded once to FP32), scaled V (flagged: 0)
+    auto stage = [&](const Raw &r, float scale, int bb, int i) {
+        float ca = 0.f, cb = 0.f, cc = 0.f;
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+        if (r.in) {
+            ca = pair_coef(r.uv.x, r.uv.y, r.sc.x, r.sc.y, d.a0h, d.a0l);
+            cb = pair_coef(r.uv.z, r.uv.w, r.sc.x, r.sc.y, d.b0h, d.b0l);
+            cc = pair_coef(r.w.x, r.w.y, r.sc.z, r.sc.w, d.csh, d.csl);
+            if (!r.flag) {
+                a = make_float4(r.a.x * scale, r.a.y * scale, r.a.z * scale, r.a.w * scale);
+                b = make_float4(r.b.x * scale, r.b.y * scale, r.b.z * scale, r.b.w * scale);
+            }
         }
-        advance(vt, vc);
+        const int at = bb * VB * 2 + (i >> 1) * 4 + (i & 1);
+        s_cb[at] = cb;
+        s_cb[at + 2] = cc;
+        s_ca[at] = ca;
+        s_ca[at + 2] = cc;
+        float *v = s_vis + bb * VB * 8 + (i >> 1) * 4 + (i & 1);     // [q][pair]
+        v[0] = a.x;
+        v[2] = a.y;
+        v[2 * VB] = a.z;
+        v[2 * VB + 2] = a.w;
+        v[4 * VB] = b.x;
+        v[4 * VB + 2] = b.y;
+        v[6 * VB] = b.z;
+        v[6 * VB + 2] = b.w;
     };
+    // the subgrid's power-of-two scale: largest unflagged |component| of V in [2^9, 2^10)
+    auto scale_exponent = [&]() {
+        float m = 0.0f;
+#pragma unroll
+        for (int w = 0; w < NPW; ++w) m = fmaxf(m, s_red[w]);
+        int e2 = 0;
+        if (m > 0.0f) frexpf(m, &e2);
+        return 10 - e2;
+    };
+    // timestep and channel (in the subgrid) of visibility k; advance() goes n visibilities on
+    struct Where {
+        int t, c, dt, dc, nc;
+        __device__ __forceinline__ Where(int k, int nc_) : t(k / nc_), c(k - t * nc_), dt(0), dc(0), nc(nc_) {}
+        __device__ __forceinline__ void step(int n) {
+            dt = n / nc;
+            dc = n - dt * nc;
+        }
+        __device__ __forceinline__ void advance() {
+            t += dt;
+            c += dc;
+            if (c >= nc) {
+                c -= nc;
+                ++t;
+            }
+        }
+    };
+    Raw raw = {};
     auto max_of = [](const float4 &a, const float4 &b) {
         return fmaxf(fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(a.z), fabsf(a.w))),
                      fmaxf(fmaxf(fabsf(b.x), fabsf(b.y)), fmaxf(fabsf(b.z), fabsf(b.w))));
     };
-    if (!mma_warp) load_batch(0);
-
     if (mma_warp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      :: "r"(smem_u32(&s_tmem)), "n"(TMEM_COLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-    } else {
+    } else if (producer) {
         // the subgrid's largest unflagged |component| (the visibilities past the first batch are
         // read here once more, for the scale; they come back from L2 when they are staged)
+        Where at(tid, d.nc);
+        load(raw, tid < kp, at.t, at.c);
         float m = 0.0f;
-        {
-            int t = vt0, c = vc0;
-            advance(t, c);
+        if (kp > VB) {
+            at.step(VB);
 #pragma unroll 4
             for (int k = VB + tid; k < kp; k += VB) {
-                const size_t vi = (bt0 + t) * g.n_chan + d.c0 + c;
+                at.advance();
+                const size_t vi = (bt0 + at.t) * g.n_chan + d.c0 + at.c;
                 const float mk = max_of(vis[2 * vi], vis[2 * vi + 1]);
                 if (!(flags && flags[vi])) m = fmaxf(m, mk);
-                advance(t, c);
             }
         }
-        if (pin && !pflag) m = fmaxf(m, max_of(pa, pb));
+        if (raw.in && !raw.flag) m = fmaxf(m, max_of(raw.a, raw.b));
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
         if (lane == 0) s_red[warp] = m;
@@ -219,6 +266,8 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
         mbar_init(smem_u32(&s_folded), NPW);
         mbar_init(smem_u32(&s_drain), 1);
         mbar_init(smem_u32(&s_atbar), 1);
+        mbar_init(smem_u32(&s_staged), 1);
+        mbar_init(smem_u32(&s_unstaged), NPW);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -272,49 +321,34 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
             }
         }
         failed = __shfl_sync(0xffffffffu, failed, 0);
+    } else if (warp == LOAD_WARP) {
+        // batches 1 .. : 32 visibilities at a time, the next ones' loads in flight; a buffer is reused
+        // once the producers are done with it
+        const float scale = ldexpf(1.0f, scale_exponent());
+        Where at(VB + lane, d.nc);
+        at.step(32);
+        if (n_batches > 1) load(raw, VB + lane < kp, at.t, at.c);
+        for (int b = 1; b < n_batches; ++b) {
+            if (b >= 2) wait_or_fail(smem_u32(&s_unstaged), (uint32_t)(b & 1), failed);
+#pragma unroll 1
+            for (int i = lane; i < VB; i += 32) {
+                const Raw r = raw;
+                at.advance();
+                load(raw, b * VB + i + 32 < kp, at.t, at.c);
+                stage(r, scale, b & 1, i);
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&s_staged));
+        }
+        if (failed && lane == 0) atomicExch(&g_sep_error, 1);
     } else {
-        // the subgrid's power-of-two scale: largest |component| of V in [2^9, 2^10)
-        float m = 0.0f;
-#pragma unroll
-        for (int w = 0; w < NPW; ++w) m = fmaxf(m, s_red[w]);
-        int e2 = 0;
-        if (m > 0.0f) frexpf(m, &e2);
-        const float scale = ldexpf(1.0f, 10 - e2), inv_scale = ldexpf(1.0f, e2 - 10);
+        const int ex = scale_exponent();
+        const float scale = ldexpf(1.0f, ex), inv_scale = ldexpf(1.0f, -ex);
         const uint32_t lane_base = tmem + ((uint32_t)(32 * yq) << 16);
         const float csig = g.c_scale, rs = 1.0f / csig;
         // FP16 hi/lo split points: A's |components| are below 2^10 sqrt(2) (integers fit FP16 up to
         // 2^11), B's at most 1 (multiples of 2^-11)
         constexpr float magic_a = 12582912.0f, magic_1 = 6144.0f;
-
-        // batch bb of the staged visibilities: phase coefficients u (f/c) k_uv - u0 k_uv and so on
-        // (float pairs, error-free products and sums, rounded once to FP32), scaled V (flagged: 0)
-        auto store_batch = [&](int bb) {
-            float ca = 0.f, cb = 0.f, cc = 0.f;
-            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-            if (pin) {
-                ca = pair_coef(puv.x, puv.y, pws.x, pws.y, d.a0h, d.a0l);
-                cb = pair_coef(puv.z, puv.w, pws.x, pws.y, d.b0h, d.b0l);
-                cc = pair_coef(pw.x, pw.y, pws.z, pws.w, d.csh, d.csl);
-                if (!pflag) {
-                    a = make_float4(pa.x * scale, pa.y * scale, pa.z * scale, pa.w * scale);
-                    b = make_float4(pb.x * scale, pb.y * scale, pb.z * scale, pb.w * scale);
-                }
-            }
-            const int at = bb * VB * 2 + (tid >> 1) * 4 + (tid & 1);
-            s_cb[at] = cb;
-            s_cb[at + 2] = cc;
-            s_ca[at] = ca;
-            s_ca[at + 2] = cc;
-            float *v = s_vis + bb * VB * 8 + (tid >> 1) * 4 + (tid & 1);     // [q][pair]
-            v[0] = a.x;
-            v[2] = a.y;
-            v[2 * VB] = a.z;
-            v[2 * VB + 2] = a.w;
-            v[4 * VB] = b.x;
-            v[4 * VB + 2] = b.y;
-            v[6 * VB] = b.z;
-            v[6 * VB + 2] = b.w;
-        };
 
         // one period's accumulator, I = S0 + i r S1 / sigma of this thread's row (polarisation
         // lane / 8, y = 8 yq + lane % 8) and its set's x, added to the image in FP32 (RN); the
@@ -428,12 +462,12 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
         f2_t X2, sx2;
         x_pair(xown, X2, sx2);
 
-        store_batch(0);
+        stage(raw, scale, 0, tid);
         producers_sync();
         int next_fold = 0;
         for (int b = 0; b < n_batches; ++b) {
             const int bb = b & 1;
-            if (b + 1 < n_batches) load_batch(b + 1);
+            if (b > 0) wait_or_fail(smem_u32(&s_staged), (uint32_t)((b - 1) & 1), failed);
             const float *cb = s_cb + bb * VB * 2, *ca = s_ca + bb * VB * 2, *vb = s_vis + bb * VB * 8;
             const int st_end = min((b + 1) * SPB, n_stages);
             // B of the stage's first (half 0) or second group (half 1); at L = 24 quarter 3 does the first
@@ -486,10 +520,8 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
                     ++next_fold;
                 }
             }
-            if (b + 1 < n_batches) {
-                store_batch(bb ^ 1);
-                producers_sync();
-            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&s_unstaged));
         }
         while (next_fold < n_periods) {
             fold(next_fold);
@@ -502,7 +534,7 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
     // the taper of this thread's epilogue pixels
     float tw_pre[PIXT];
 #pragma unroll
-    for (int i = 0; i < PIXT; ++i) tw_pre[i] = !mma_warp && tid + i * NP < SPIX ? taper[tid + i * NP] : 0.0f;
+    for (int i = 0; i < PIXT; ++i) tw_pre[i] = producer && tid + i * NP < SPIX ? taper[tid + i * NP] : 0.0f;
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     if (!__syncthreads_or(failed)) {
         if (aterms) {
@@ -511,7 +543,7 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
             if (late) atomicExch(&g_sep_error, 1);
         }
         // image-domain kernel per pixel: taper * A_p^H I A_q (with the centring factor when FUSED)
-        if (!mma_warp) {
+        if (producer) {
 #pragma unroll
             for (int ip = 0; ip < PIXT; ++ip) {
                 const int pix = tid + ip * NP;
