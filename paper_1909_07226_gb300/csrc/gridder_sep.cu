@@ -101,9 +101,6 @@ struct SepG {
     static constexpr int CB_OFF = B_OFF + 4 * B_STAGE, CA_OFF = CB_OFF + 2 * VB * 8;
     static constexpr int VIS_OFF = CA_OFF + 2 * VB * 8;
     static constexpr int SMEM = VIS_OFF + 2 * VB * 32;
-    // the subgrid's A-terms after the main loop: [2 stations][L^2] 2 x 2 complex, over B and the batches
-    static constexpr int AT_OFF = B_OFF;
-    static constexpr uint32_t AT_BYTES = SPIX * 32;
     // accumulator: main (m, re/im, x) at 0 .. 4 L, correction (m = 0) at 4 L .. 6 L; then the
     // sets' A, 32 columns each (group i at + 16 i: 8 columns hi, 8 lo)
     static constexpr uint32_t A_COL = 6 * L;
@@ -112,7 +109,6 @@ struct SepG {
     static constexpr int PIXT = (SPIX + NP - 1) / NP;            // pixels per producer in the epilogue
     static_assert(L == 32 || L == 24 || L == 16, "subgrid sizes of the separable kernels");
     static_assert(CTAS * (SMEM + 2048) <= 227 * 1024, "shared memory of the SM's CTAs");
-    static_assert(AT_OFF % 16 == 0 && AT_OFF + 2 * (int)AT_BYTES <= SMEM, "A-terms over B and the batches");
     static_assert(B_OFF % 128 == 0 && CB_OFF % 16 == 0, "alignment of the B tiles and the batches");
     static_assert(A_COL % 16 == 0 && A_COL + 2 * 16 * SG <= TMEM_COLS, "tensor memory");
 };
@@ -129,15 +125,15 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
                                                  float4 *__restrict__ o) {
     using C = SepG<L>;
     constexpr int SL = C::SL, SPIX = C::SPIX, NQ = C::NQ, B_GROUP = C::B_GROUP, B_STAGE = C::B_STAGE;
-    constexpr int FFT_P = C::FFT_P, FFT_S = C::FFT_S, AT_OFF = C::AT_OFF, XS = C::XS, PIXT = C::PIXT;
-    constexpr uint32_t AT_BYTES = C::AT_BYTES, A_COL = C::A_COL;
+    constexpr int FFT_P = C::FFT_P, FFT_S = C::FFT_S, XS = C::XS, PIXT = C::PIXT;
+    constexpr uint32_t A_COL = C::A_COL;
     extern __shared__ __align__(1024) uint8_t smem[];
     float2 *s_img = (float2 *)smem;                 // 4 planes [L][L + 1]
     uint8_t *sB = smem + C::B_OFF;
     float *s_cb = (float *)(smem + C::CB_OFF), *s_ca = (float *)(smem + C::CA_OFF);
     float *s_vis = (float *)(smem + C::VIS_OFF);
     __shared__ uint32_t s_tmem;
-    __shared__ __align__(8) uint64_t s_full[2], s_empty[2], s_foldbar, s_folded, s_drain, s_atbar,
+    __shared__ __align__(8) uint64_t s_full[2], s_empty[2], s_foldbar, s_folded, s_drain,
         s_staged, s_unstaged;
     __shared__ float s_red[NPW];
 
@@ -265,7 +261,6 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
         mbar_init(smem_u32(&s_foldbar), 1);
         mbar_init(smem_u32(&s_folded), NPW);
         mbar_init(smem_u32(&s_drain), 1);
-        mbar_init(smem_u32(&s_atbar), 1);
         mbar_init(smem_u32(&s_staged), 1);
         mbar_init(smem_u32(&s_unstaged), NPW);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -275,7 +270,20 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = s_tmem;
 
-    bool failed = false, at_issued = false;
+    bool failed = false;
+    // the epilogue's A-terms of a producer's pixel ip (A_p, A_q), read straight from L2: the first
+    // AHEAD pixels' before the last fold, whose wait covers them, each later pixel's when an
+    // earlier one has been used
+    constexpr int AHEAD = PIXT < 2 ? PIXT : 2;
+    M22 Ap[AHEAD], Aq[AHEAD];
+    auto load_aterms = [&](int ip) {
+        const int pix = tid + ip * NP;
+        if (aterms && pix < SPIX) {
+            const float4 *base = aterms + 2 * ((size_t)d.slot * g.n_stations) * SPIX + 2 * pix;
+            Ap[ip % AHEAD] = load_m22(base + 2 * (size_t)d.st_p * SPIX);
+            Aq[ip % AHEAD] = load_m22(base + 2 * (size_t)d.st_q * SPIX);
+        }
+    };
     const int yq = warp & 3, set = (warp >> 2) & 1;   // lane quarter (rows 32 yq ..) and producer set
 
     if (mma_warp) {
@@ -309,16 +317,6 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
             bool late = false;
             wait_or_fail(smem_u32(&s_drain), 0u, late);     // bounded: let own MMAs finish before the free
             if (late) failed = true;
-            // the tensor cores are done with the stage buffers: bring the subgrid's A-terms (A_p,
-            // A_q) into them while the producers fold
-            if (aterms && !failed) {
-                const float4 *base = aterms + 2 * ((size_t)d.slot * g.n_stations) * SPIX;
-                mbar_expect_tx(smem_u32(&s_atbar), 2 * AT_BYTES);
-                bulk_g2s(smem_u32(smem + AT_OFF), base + 2 * (size_t)d.st_p * SPIX, AT_BYTES, smem_u32(&s_atbar));
-                bulk_g2s(smem_u32(smem + AT_OFF + AT_BYTES), base + 2 * (size_t)d.st_q * SPIX, AT_BYTES,
-                         smem_u32(&s_atbar));
-                at_issued = true;
-            }
         }
         failed = __shfl_sync(0xffffffffu, failed, 0);
     } else if (warp == LOAD_WARP) {
@@ -523,6 +521,8 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&s_unstaged));
         }
+#pragma unroll
+        for (int ip = 0; ip < AHEAD; ++ip) load_aterms(ip);
         while (next_fold < n_periods) {
             fold(next_fold);
             ++next_fold;
@@ -537,11 +537,6 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
     for (int i = 0; i < PIXT; ++i) tw_pre[i] = producer && tid + i * NP < SPIX ? taper[tid + i * NP] : 0.0f;
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     if (!__syncthreads_or(failed)) {
-        if (aterms) {
-            bool late = false;
-            wait_or_fail(smem_u32(&s_atbar), 0u, late);
-            if (late) atomicExch(&g_sep_error, 1);
-        }
         // image-domain kernel per pixel: taper * A_p^H I A_q (with the centring factor when FUSED)
         if (producer) {
 #pragma unroll
@@ -559,12 +554,8 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
                     for (int c = 0; c < 4; ++c)
                         P.m[c] = make_float2(P.m[c].x * cs - P.m[c].y * sn, P.m[c].x * sn + P.m[c].y * cs);
                 }
-                if (aterms) {
-                    const float4 *at = (const float4 *)(smem + AT_OFF);
-                    const M22 Ap = load_m22(at + 2 * pix);
-                    const M22 Aq = load_m22(at + 2 * (SPIX + pix));
-                    P = herm_mul_mul(Ap, P, Aq);
-                }
+                if (aterms) P = herm_mul_mul(Ap[ip % AHEAD], P, Aq[ip % AHEAD]);
+                if (ip + AHEAD < PIXT) load_aterms(ip + AHEAD);
                 if (FUSED) {
                     const float tw = tw_pre[ip] * (1.0f / SPIX);      // with the transform's L^-2
 #pragma unroll
@@ -598,10 +589,6 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
         }
     }
     __syncthreads();
-    if (at_issued) {      // the copies have landed before the CTA's shared memory is released
-        bool late = false;
-        wait_or_fail(smem_u32(&s_atbar), 0u, late);
-    }
     if (mma_warp)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "n"(TMEM_COLS));
 }
