@@ -250,9 +250,22 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
             float2 *dst = (float2 *)smem + ln * C::PIX_P + pol;
             fft_line<SL, +1>([&](int n) { return row[n]; }, [&](int k, float2 v) { dst[4 * k] = v; });
         }
-        __syncthreads();
     }
-    M22 P[C::TPW];
+    // the A-terms of this thread's pixels, two pixels ahead
+    constexpr int AHEAD = C::TPW < 2 ? C::TPW : 2;
+    M22 P[C::TPW], Ap[AHEAD], Aq[AHEAD];
+    auto load_aterms = [&](int i) {
+        const int tile = warp + NWW * i;
+        if (aterms && warp < NWW && tile < C::NTILE) {
+            const int y = 8 * (tile / (SL / 4)) + (lane >> 2), x = 4 * (tile % (SL / 4)) + (lane & 3);
+            const float4 *base = aterms + 2 * ((size_t)d.slot * g.n_stations) * SPIX + 2 * (y * SL + x);
+            Ap[i % AHEAD] = load_m22(base + 2 * (size_t)d.st_p * SPIX);
+            Aq[i % AHEAD] = load_m22(base + 2 * (size_t)d.st_q * SPIX);
+        }
+    };
+#pragma unroll
+    for (int i = 0; i < AHEAD; ++i) load_aterms(i);
+    if (FUSED) __syncthreads();
     if (warp < NWW) {
         float m = 0.0f;
 #pragma unroll
@@ -268,12 +281,8 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
                 for (int q = 0; q < 4; ++q)
                     P[i].m[q] = make_float2(P[i].m[q].x * cs + P[i].m[q].y * sn, P[i].m[q].y * cs - P[i].m[q].x * sn);
             }
-            if (aterms) {
-                const float4 *base = aterms + 2 * ((size_t)d.slot * g.n_stations) * SPIX + 2 * pix;
-                const M22 Ap = load_m22(base + 2 * (size_t)d.st_p * SPIX);
-                const M22 Aq = load_m22(base + 2 * (size_t)d.st_q * SPIX);
-                P[i] = mul_mul_herm(Ap, P[i], Aq);
-            }
+            if (aterms) P[i] = mul_mul_herm(Ap[i % AHEAD], P[i], Aq[i % AHEAD]);
+            if (i + AHEAD < C::TPW) load_aterms(i + AHEAD);
             const float tw = FUSED ? taper[pix] * (1.0f / SPIX) : taper[pix];      // with the transform's L^-2
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
