@@ -333,6 +333,7 @@ def load_tuning(path: str) -> bool:
 class Plan:
     handle: ctypes.c_void_p
     stats: PlanStats
+    shapes: Optional[dict] = None      # buffer shapes, from the (fixed) stats at the first call
 
     @property
     def n_subgrids(self):
@@ -395,35 +396,50 @@ def plan_from_workload(wl, **opt) -> Plan:
 # ---------------------------------------------------------------------------
 # device-buffer calls (torch CUDA tensors)
 
+# The calls below cost a small plan's GPU time on the host (a gridding of a hundred subgrids is
+# about 10 us on both sides), so the checks are kept lean: shapes are made once per plan,
+# torch is looked up once, and pointers go to ctypes as plain integers.
+
+_torch = None
+
+
+def _import_torch():
+    global _torch
+    if _torch is None:
+        import torch
+        _torch = torch
+    return _torch
+
+
 def _dptr(t, name, dtype=None, shape=None, optional=False):
     if t is None:
         if optional:
             return None
         raise ValueError(f"{name} is required")
-    import torch
-    if not isinstance(t, torch.Tensor) or not t.is_cuda:
+    if not isinstance(t, _import_torch().Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
     if dtype is not None and t.dtype != dtype:
         raise TypeError(f"{name} must have dtype {dtype}, got {t.dtype}")
-    if shape is not None and tuple(t.shape) != tuple(shape):
+    if shape is not None and t.shape != shape:
         raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream(stream):
-    import torch
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+        stream = _import_torch().cuda.current_stream()
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _shapes(plan: Plan):
-    s = plan.stats
-    L, N = s.subgrid_size, s.grid_size
-    return dict(vis=(s.n_bl, s.n_t, s.n_chan, 4), flags=(s.n_bl, s.n_t, s.n_chan),
-                aterms=(s.n_slots, s.n_stations, L, L, 4), taper=(L, L), grid=(s.n_w_layers, N, N, 4))
+    if plan.shapes is None:
+        s = plan.stats
+        L, N = s.subgrid_size, s.grid_size
+        plan.shapes = dict(vis=(s.n_bl, s.n_t, s.n_chan, 4), flags=(s.n_bl, s.n_t, s.n_chan),
+                           aterms=(s.n_slots, s.n_stations, L, L, 4), taper=(L, L), grid=(s.n_w_layers, N, N, 4))
+    return plan.shapes
 
 
 def grid(plan: Plan, vis, flags, aterms, taper, grid_out, stream=None):
