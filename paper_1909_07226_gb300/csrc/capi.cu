@@ -36,6 +36,13 @@ idg_status launch_subgrid_fft(const idg_plan *p, int64_t count, int direction, v
     return launch_fft(p->L, count, direction, subgrids, stream);
 }
 
+// L = 32 only: variant 0 of the other sizes is the packed-FP32 gridder.  Against separate gridder
+// and transform launches this saves the transform's pass over the scratch (64 B per pixel).
+bool gridder_transforms(const idg_plan *p, const Geometry &g) {
+    return g.L == 32 && g.separable && !g.recurrence && p->kernel_variant(IDG_KERNEL_GRIDDER) == 0 &&
+           p->opts.fft_mode == IDG_FFT_FP32;
+}
+
 // One stream-ordered memory pool per device for the subgrid scratch, kept
 // alive (release threshold = max) so repeated calls do not return memory to
 // the driver between steps.
@@ -1068,11 +1075,13 @@ static idg_status grid_part(const idg_plan *p, const Geometry &g, Order o, int64
     for (int64_t f = first; f < first + count && st == IDG_OK; f += chunk) {
         const int64_t cnt = std::min(chunk, first + count - f);
         const SubgridSet set = order_of(p, o, f, cnt);
+        const bool one = gridder_transforms(p, g);
         {
             ProfileScope ps(IDG_KERNEL_GRIDDER, s, vispix(p, f, cnt, o));
-            st = launch_gridder(g, set, p->kernel_variant(IDG_KERNEL_GRIDDER), vis, flags, aterms, taper, scratch, s);
+            st = one ? launch_gridder_sep_transform(g, set, vis, flags, aterms, taper, scratch, s)
+                     : launch_gridder(g, set, p->kernel_variant(IDG_KERNEL_GRIDDER), vis, flags, aterms, taper, scratch, s);
         }
-        if (st == IDG_OK) {
+        if (st == IDG_OK && !one) {
             ProfileScope ps(IDG_KERNEL_FFT, s, (double)cnt);
             st = launch_subgrid_fft(p, cnt, -1, scratch, s);
         }

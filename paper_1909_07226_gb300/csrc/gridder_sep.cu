@@ -115,15 +115,19 @@ struct SepG {
 
 __device__ __forceinline__ void producers_sync() { asm volatile("bar.sync 1, %0;" :: "n"(NP) : "memory"); }
 
-// One subgrid d of geometry g (taper and A-terms applied): into o[L][L][4], or with
-// FUSED transformed in shared memory and added into the grid o[layer][N][N][4]
-// (Algorithm 1: direct sum, image-domain kernel, "FFT", add to the master grid).
-template <int L, bool FUSED>
+// What a launch leaves: subgrid images o[L][L][4] (taper and A-terms applied), their transforms
+// in the same place, or the transforms added into the grid o[layer][N][N][4]
+enum Out { kImage, kTransform, kGrid };
+
+// One subgrid d of geometry g (Algorithm 1: direct sum, image-domain kernel, "FFT", add to the
+// master grid)
+template <int L, Out OUT>
 __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSubgrid d,
                                                  const float4 *__restrict__ vis, const uint8_t *__restrict__ flags,
                                                  const float4 *__restrict__ aterms, const float *__restrict__ taper,
                                                  float4 *__restrict__ o) {
     using C = SepG<L>;
+    constexpr bool FUSED = OUT != kImage;       // transformed here
     constexpr int SL = C::SL, SPIX = C::SPIX, NQ = C::NQ, B_GROUP = C::B_GROUP, B_STAGE = C::B_STAGE;
     constexpr int FFT_P = C::FFT_P, FFT_S = C::FFT_S, XS = C::XS, PIXT = C::PIXT;
     constexpr uint32_t A_COL = C::A_COL;
@@ -581,10 +585,14 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
             }
             __syncthreads();
             if (tid < 4 * SL) {
-                float2 *dst = (float2 *)o + ((((size_t)d.layer * g.N + d.r0) * g.N + d.q0 + ln) * 4 + pol);
-                const size_t pitch = (size_t)g.N * 4;
+                const size_t corner = OUT == kGrid ? ((size_t)d.layer * g.N + d.r0) * g.N + d.q0 : 0;
+                const size_t pitch = 4 * (OUT == kGrid ? (size_t)g.N : (size_t)SL);
+                float2 *dst = (float2 *)o + (corner + ln) * 4 + pol;
                 fft_line<SL, -1>([&](int n) { return plane[n * FFT_P + ln]; },
-                                 [&](int k, float2 v) { red_add_f2(dst + k * pitch, v); });
+                                 [&](int k, float2 v) {
+                                     if (OUT == kGrid) red_add_f2(dst + k * pitch, v);
+                                     else dst[k * pitch] = v;
+                                 });
             }
         }
     }
@@ -593,14 +601,14 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "n"(TMEM_COLS));
 }
 
-// one CTA per subgrid of one plan (plan index idx[b] or first + b): subgrid images
-template <int L>
+// one CTA per subgrid of one plan (plan index idx[b] or first + b): subgrid images or transforms
+template <int L, Out OUT>
 __global__ void __launch_bounds__(NT, CTAS)
 gridder_sep_kernel(Geometry g, const int32_t *__restrict__ idx, int64_t first, const float4 *__restrict__ vis,
                    const uint8_t *__restrict__ flags, const float4 *__restrict__ aterms,
                    const float *__restrict__ taper, float4 *__restrict__ out) {
     const int sid = idx ? idx[blockIdx.x] : (int)(first + blockIdx.x);
-    gridder_sep_body<L, false>(g, g.sub[sid], vis, flags, aterms, taper, out + (size_t)blockIdx.x * L * L * 2);
+    gridder_sep_body<L, OUT>(g, g.sub[sid], vis, flags, aterms, taper, out + (size_t)blockIdx.x * L * L * 2);
 }
 
 // fused: one CTA per subgrid, transformed and added into the grid
@@ -611,20 +619,22 @@ gridder_sep_fused_kernel(Geometry g, const int32_t *__restrict__ idx, int64_t fi
                          const float *__restrict__ taper, float4 *__restrict__ grid) {
     allow_dependents();
     const int sid = idx ? idx[blockIdx.x] : (int)(first + blockIdx.x);
-    gridder_sep_body<L, true>(g, g.sub[sid], vis, flags, aterms, taper, grid);
+    gridder_sep_body<L, kGrid>(g, g.sub[sid], vis, flags, aterms, taper, grid);
     complete_after_primary();
 }
 
 template <int L>
-idg_status launch_sep_set(bool fused, const Geometry &g, const SubgridSet &set, const void *vis, const uint8_t *flags,
+idg_status launch_sep_set(Out out_kind, const Geometry &g, const SubgridSet &set, const void *vis, const uint8_t *flags,
                           const void *aterms, const float *taper, void *out, cudaStream_t s) {
-    auto kern = fused ? gridder_sep_fused_kernel<L> : gridder_sep_kernel<L>;
+    auto kern = out_kind == kGrid        ? gridder_sep_fused_kernel<L>
+                : out_kind == kTransform ? gridder_sep_kernel<L, kTransform>
+                                         : gridder_sep_kernel<L, kImage>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SepG<L>::SMEM);
     if (e != cudaSuccess) return cuda_fail(e, "separable gridder smem attribute");
     kern<<<(unsigned)set.count, NT, SepG<L>::SMEM, s>>>(g, set.idx, set.first, (const float4 *)vis, flags,
                                                        (const float4 *)aterms, taper, (float4 *)out);
     e = cudaGetLastError();
-    return e == cudaSuccess ? IDG_OK : cuda_fail(e, fused ? "separable fused gridder launch" : "separable gridder launch");
+    return e == cudaSuccess ? IDG_OK : cuda_fail(e, out_kind == kGrid ? "separable fused gridder launch" : "separable gridder launch");
 }
 
 }  // namespace
@@ -662,28 +672,31 @@ idg_status launch_gridder_sep_job(const Geometry &g, const SubgridSet &set, cons
     return e == cudaSuccess ? IDG_OK : cuda_fail(e, "separable gridder job launch");
 }
 
-idg_status launch_gridder_sep(const Geometry &g, const SubgridSet &set, const void *vis, const uint8_t *flags,
-                              const void *aterms, const float *taper, void *out, void *stream) {
+static idg_status launch_sep_any(Out kind, const Geometry &g, const SubgridSet &set, const void *vis, const uint8_t *flags,
+                                 const void *aterms, const float *taper, void *out, void *stream) {
     if (!separable_size(g.L) || !g.separable)
         return fail(IDG_ERR_UNSUPPORTED, "the separable gridder needs L = 32, 24 or 16 and a separable plan");
     if (set.count <= 0) return IDG_OK;
     switch (g.L) {
-    case 32: return launch_sep_set<32>(false, g, set, vis, flags, aterms, taper, out, (cudaStream_t)stream);
-    case 24: return launch_sep_set<24>(false, g, set, vis, flags, aterms, taper, out, (cudaStream_t)stream);
-    default: return launch_sep_set<16>(false, g, set, vis, flags, aterms, taper, out, (cudaStream_t)stream);
+    case 32: return launch_sep_set<32>(kind, g, set, vis, flags, aterms, taper, out, (cudaStream_t)stream);
+    case 24: return launch_sep_set<24>(kind, g, set, vis, flags, aterms, taper, out, (cudaStream_t)stream);
+    default: return launch_sep_set<16>(kind, g, set, vis, flags, aterms, taper, out, (cudaStream_t)stream);
     }
+}
+
+idg_status launch_gridder_sep(const Geometry &g, const SubgridSet &set, const void *vis, const uint8_t *flags,
+                              const void *aterms, const float *taper, void *out, void *stream) {
+    return launch_sep_any(kImage, g, set, vis, flags, aterms, taper, out, stream);
+}
+
+idg_status launch_gridder_sep_transform(const Geometry &g, const SubgridSet &set, const void *vis, const uint8_t *flags,
+                                        const void *aterms, const float *taper, void *out, void *stream) {
+    return launch_sep_any(kTransform, g, set, vis, flags, aterms, taper, out, stream);
 }
 
 idg_status launch_gridder_sep_fused(const Geometry &g, const SubgridSet &set, const void *vis, const uint8_t *flags,
                                     const void *aterms, const float *taper, void *grid, void *stream) {
-    if (!separable_size(g.L) || !g.separable)
-        return fail(IDG_ERR_UNSUPPORTED, "the separable gridder needs L = 32, 24 or 16 and a separable plan");
-    if (set.count <= 0) return IDG_OK;
-    switch (g.L) {
-    case 32: return launch_sep_set<32>(true, g, set, vis, flags, aterms, taper, grid, (cudaStream_t)stream);
-    case 24: return launch_sep_set<24>(true, g, set, vis, flags, aterms, taper, grid, (cudaStream_t)stream);
-    default: return launch_sep_set<16>(true, g, set, vis, flags, aterms, taper, grid, (cudaStream_t)stream);
-    }
+    return launch_sep_any(kGrid, g, set, vis, flags, aterms, taper, grid, stream);
 }
 
 idg_status read_sep_error(int *code) {

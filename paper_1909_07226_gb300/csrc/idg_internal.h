@@ -250,6 +250,9 @@ constexpr int32_t kSepFusedKpMin = 64;
 // with the transform and the adder into grid
 idg_status launch_gridder_sep(const Geometry &g, const SubgridSet &set, const void *vis, const uint8_t *flags,
                               const void *aterms, const float *taper, void *out, void *stream);
+// the same images transformed in the kernel (image -> uv, as launch_fft with direction -1)
+idg_status launch_gridder_sep_transform(const Geometry &g, const SubgridSet &set, const void *vis, const uint8_t *flags,
+                                        const void *aterms, const float *taper, void *out, void *stream);
 idg_status launch_gridder_sep_fused(const Geometry &g, const SubgridSet &set, const void *vis, const uint8_t *flags,
                                     const void *aterms, const float *taper, void *grid, void *stream);
 idg_status read_sep_error(int *code);
@@ -330,6 +333,10 @@ idg_status read_classical_error(int *code);
 bool dft_tc_supported(int L);
 idg_status launch_dft_tc(int L, int64_t count, int direction, void *subgrids, void *stream);
 idg_status read_dft_error(int *code);
+// whether the unfused gridding takes gridder and transform in one launch
+// (launch_gridder_sep_transform): the plan's gridder is the separable one (g: the launch's
+// geometry) and its transform the FP32 one
+bool gridder_transforms(const idg_plan *p, const Geometry &g);
 // the plan's transform (FP32 shared-memory FFT or the tensor-core form)
 idg_status launch_subgrid_fft(const idg_plan *p, int64_t count, int direction, void *subgrids, void *stream);
 

@@ -101,8 +101,12 @@ extern "C" idg_status idg_grid_no_alloc(const idg_plan *p, const void *vis, cons
     const bool sorted = p->opts.adder_mode == IDG_ADDER_SORTED;
     const SubgridSet all = sorted ? SubgridSet{nullptr, 0, n, p->kp_plan.data()}
                                   : SubgridSet{p->d_order, 0, n, p->kp_order.data()};
-    st = launch_gridder(g, all, p->kernel_variant(IDG_KERNEL_GRIDDER), vis, flags, aterms, taper, scratch, s);
-    if (st == IDG_OK) st = launch_subgrid_fft(p, n, -1, scratch, s);
+    if (gridder_transforms(p, g)) {
+        st = launch_gridder_sep_transform(g, all, vis, flags, aterms, taper, scratch, s);
+    } else {
+        st = launch_gridder(g, all, p->kernel_variant(IDG_KERNEL_GRIDDER), vis, flags, aterms, taper, scratch, s);
+        if (st == IDG_OK) st = launch_subgrid_fft(p, n, -1, scratch, s);
+    }
     if (st == IDG_OK)
         st = sorted ? launch_adder_sorted(g, all, scratch, grid,
                                           SortedTiles{p->d_tile_ids, p->d_tile_first, p->d_tile_sub, p->n_tiles_sorted,
