@@ -360,8 +360,9 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             constexpr int XC = C::XC;
             if (yq < NQ) {
-                const int y = 8 * yq + (lane & 7);
-                float2 *img = s_img + (lane >> 3) * FFT_S + y * FFT_P + set * XS;
+                // row 8 a + b: polarisation 2 (b / 4) + a / 2, y = 4 (a % 2) + b % 4 of the block
+                const int y = 8 * yq + 4 * ((lane >> 3) & 1) + (lane & 3), q = 2 * ((lane >> 2) & 1) + (lane >> 4);
+                float2 *img = s_img + q * FFT_S + y * FFT_P + set * XS;
                 const float *rp = g.sep + 2 * SL + y * SL + set * XS;
 #pragma unroll
                 for (int x0 = 0; x0 < XS; x0 += XC) {
@@ -402,26 +403,36 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
 
         // A entries: lane = 4 ylo + jp forms Ey of row y = 8 yq + ylo for visibilities 2 jp and 2 jp + 1
         // of a group and multiplies the four polarisations with it (16 x 256-bit fragments)
-        const int jp = lane & 3;
-        const float Yv = (float)(8 * yq + (lane >> 2) - SL / 2);
-        const float ty = yq < NQ ? g.sep[SL + 8 * yq + (lane >> 2)] : 0.0f;
-        const f2_t Y2 = f2_pack(Yv, Yv), ty2 = f2_pack(ty, ty);
+        const int jp = lane & 3, qh = lane >> 4;
+        const int y0 = 8 * yq + ((lane >> 2) & 3);
+        const float Yv = (float)(y0 - SL / 2);
+        const f2_t Y2[2] = {f2_bcast(Yv), f2_bcast(Yv + 4.0f)};
+        const f2_t ty2[2] = {f2_bcast(yq < NQ ? g.sep[SL + y0] : 0.0f), f2_bcast(yq < NQ ? g.sep[SL + y0 + 4] : 0.0f)};
         auto a_unit = [&](const float *cb, const float *vb, int pair, uint32_t (&e)[16]) {
             const ulonglong2 cf = *(const ulonglong2 *)(cb + 4 * (pair + jp));
-            float p0, p1, sn0, cs0, sn1, cs1;
-            f2_unpack(f2_fma(cf.y, ty2, f2_mul(cf.x, Y2)), p0, p1);
-            __sincosf(p0, &sn0, &cs0);
-            __sincosf(p1, &sn1, &cs1);
-            const f2_t c2 = f2_pack(cs0, cs1), s2 = f2_pack(sn0, sn1), n2 = f2_mul(s2, f2_bcast(-1.0f));
+            f2_t c2[2], s2[2], n2[2];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const ulonglong2 v = *(const ulonglong2 *)(vb + 2 * VB * q + 4 * (pair + jp));
-                f2_t hr, lr, hi, li;
-                f2_split(f2_fma(v.y, n2, f2_mul(v.x, c2)), magic_a, hr, lr);
-                f2_split(f2_fma(v.y, c2, f2_mul(v.x, s2)), magic_a, hi, li);
-                const int k = 8 * (q >> 1) + 2 * (q & 1);
-                pack_pairs(hr, hi, e[k], e[k + 1]);
-                pack_pairs(lr, li, e[k + 4], e[k + 5]);
+            for (int h = 0; h < 2; ++h) {
+                float p0, p1, sn0, cs0, sn1, cs1;
+                f2_unpack(f2_fma(cf.y, ty2[h], f2_mul(cf.x, Y2[h])), p0, p1);
+                __sincosf(p0, &sn0, &cs0);
+                __sincosf(p1, &sn1, &cs1);
+                c2[h] = f2_pack(cs0, cs1);
+                s2[h] = f2_pack(sn0, sn1);
+                n2[h] = f2_mul(s2[h], f2_bcast(-1.0f));
+            }
+#pragma unroll
+            for (int ql = 0; ql < 2; ++ql) {
+                const ulonglong2 v = *(const ulonglong2 *)(vb + 2 * VB * (2 * qh + ql) + 4 * (pair + jp));
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    f2_t hr, lr, hi, li;
+                    f2_split(f2_fma(v.y, n2[h], f2_mul(v.x, c2[h])), magic_a, hr, lr);
+                    f2_split(f2_fma(v.y, c2[h], f2_mul(v.x, s2[h])), magic_a, hi, li);
+                    const int k = 8 * ql + 2 * h;
+                    pack_pairs(hr, hi, e[k], e[k + 1]);
+                    pack_pairs(lr, li, e[k + 4], e[k + 5]);
+                }
             }
         };
         // B entries of 8 pixel columns from 8 xblk for one group: lane = 8 jl + (x % 8), visibilities
@@ -435,16 +446,17 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
             f2_unpack(f2_fma(cf.y, sx2, f2_mul(cf.x, X2)), p0, p1);
             __sincosf(p0, &sn0, &cs0);
             __sincosf(p1, &sn1, &cs1);
-            const f2_t c2 = f2_pack(cs0, cs1), s2 = f2_pack(sn0, sn1), n2 = f2_mul(s2, f2_bcast(-1.0f));
+            const f2_t c2 = f2_pack(cs0, cs1), s2 = f2_pack(sn0, sn1);
             const f2_t cz = f2_mul(cf.y, f2_pack(csig, csig)), zc = f2_mul(cz, c2), zs = f2_mul(cz, s2);
             f2_t hc, lc, hs, ls, hn, ln;
             f2_split(c2, magic_1, hc, lc);
             f2_split(s2, magic_1, hs, ls);
-            f2_split(n2, magic_1, hn, ln);
+            hn = f2_mul(hs, f2_bcast(-1.0f));
+            ln = f2_mul(ls, f2_bcast(-1.0f));
             uint32_t w[6][2];
             pack_pairs(hc, hn, w[0][0], w[0][1]);
             pack_pairs(hs, hc, w[1][0], w[1][1]);
-            pack_pairs(zc, f2_mul(cz, n2), w[2][0], w[2][1]);
+            pack_pairs(zc, f2_mul(zs, f2_bcast(-1.0f)), w[2][0], w[2][1]);
             pack_pairs(zs, zc, w[3][0], w[3][1]);
             pack_pairs(lc, ln, w[4][0], w[4][1]);
             pack_pairs(ls, lc, w[5][0], w[5][1]);
