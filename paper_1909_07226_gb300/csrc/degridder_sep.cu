@@ -11,35 +11,48 @@
 //   Ex*_k(x) = exp(-i (a_k X + c_k s(x))),  Ey*_k(y) = exp(-i (b_k Y + c_k t(y))).
 // Both terms are one complex matrix product on the tensor cores,
 //   T_kq(y) = sum_x Ex*_k(x) Q0_q(x, y) + sum_x (-i c_k Ex*_k(x)) Q1_q(x, y),
-// with rows (re/im, visibility) of a tile of 64 visibilities, columns (q, y),
-// 128 of them, and K = (x, re/im) twice (m = 0, then m = 1).  The sum over y
-// with the visibility's own phasors, y_kq = sum_y Ey*_k(y) T_kq(y), runs on
-// the CUDA cores (FP32, round to nearest), one thread per tile row.
+// with rows the 128 visibilities of a tile, columns (q, y, re/im) and K = (x, cos/sin)
+// twice (m = 0, then m = 1).  The sum over y with the visibility's own phasors,
+// y_kq = sum_y Ey*_k(y) T_kq(y), runs on the CUDA cores (FP32, round to nearest).
 //
-// GEMM.  A holds the real 2 x 2 embedding of a = Ex*_k(x) (m = 0) and of
-// a = -i c_k sigma Ex*_k(x) (m = 1, sigma a power of two with max |c| sigma
-// <= 1): row k (re) = (Re a, -Im a), row 64 + k (im) = (Im a, Re a) over
-// K = (x, re/im).  B[(q, y)] = (Re, Im) of Q0 = s P and of Q1 = s r P / sigma
-// (s a power of two per subgrid), so both products carry the same scale.  The
-// m = 0 operands are split into FP16 hi + lo and take A_hi B_hi + A_hi B_lo +
-// A_lo B_hi; the m = 1 term (at most theta relative) takes A_hi B_hi.  Per K
-// step of 16 (8 x): four MMAs of N = 128.  The accumulation is 16 MMAs long,
-// so no folds are needed.
+// GEMM.  A holds (cos, sin) of Ex_k(x) (m = 0) and c sigma (-sin, cos) (m = 1, sigma a
+// power of two with max |c| sigma <= 1), one tensor-memory row per visibility; B holds
+// the 2 x 2 real embedding of Q0 = s P and of Q1 = s r P / sigma (s a power of two per
+// subgrid): row re of (q, y) is (Re Q, Im Q), row im (Im Q, -Re Q).  The embedding sits
+// on the image side, where it is formed once per subgrid, not per visibility.  The
+// m = 0 operands are split into FP16 hi + lo (A's hi a multiple of 2^-11) and take
+// A_hi B_hi + A_hi B_lo + A_lo B_hi; the m = 1 term (at most theta relative) takes
+// A_hi B_hi.  Per K step of 16 (8 x): four MMAs of N = 128 (96 at L = 24) for two of
+// the four polarisations, then the same for the other two (all four at L = 16).  The
+// accumulation is 16 MMAs long, so no folds are needed.
 //
-// Schedule.  One CTA per subgrid, one CTA per SM.  All warps first form the
-// image (split from the grid and inverse transform in shared memory when
-// FUSED, while two bulk copies bring the subgrid's A-terms), the corrections,
-// the scale and B (shared memory, fixed for the subgrid).  Then per tile: a
-// coefficient warp stages the visibilities' phase coefficients (float pairs,
-// error-free FP32 products and sums); eight producer warps write A (shared
-// memory, one core matrix per warp store); the consumers form the tile's Ey*
-// table while its MMAs run;
-// the MMA warp issues the 16 MMAs into one of four accumulators; eight consumer
-// warps read their rows' columns, sum over y, pair the re and im rows of each
-// visibility through shared memory and write the visibilities.  The A stages
-// (two, freed by the MMAs) and the coefficient and accumulator stages (four,
-// freed by the consumers) are separate, so producers, MMAs and consumers
-// overlap across tiles.  Tensor memory: accumulator e at 128 e.
+// Schedule.  One CTA per subgrid, two CTAs per SM (256 tensor-memory columns and 105 KB of
+// shared memory each): the prologue of one, and the sums of one, run under the other's
+// MMAs.  The prologue brings the grid rows by bulk copy, transforms them (one thread per
+// line and polarisation), applies A-terms and taper in registers and writes B.  Then per
+// tile a visibility belongs to two threads (warps w and w + 4): each forms A for half of
+// the x and the y phasors and the sum for half of the y; the two meet through shared
+// memory, each finishing two polarisations.  A ninth warp issues the MMAs.  The phase
+// coefficients of the next tile are formed while the last part's MMAs run, the outputs
+// of a tile and its Ey* while the first part's do.  X, s(x) and t(y) are kernel-parameter
+// constants: tables in shared memory cost 430 of 919 wavefronts per tile.
+// Tensor memory: accumulator at 0, A at 128 (hi, lo and m = 1, a column per x).
+//
+// What bounds it, and what the choices measured (LOFAR-like plan of 45.9 k subgrids of about
+// 1600 visibilities, 73.9 M; and A-terms every 16 s, 18.4 M in 89.4 k of about 206):
+//   one CTA per SM, embedding on the visibility side, Ey
+//   table and re/im exchange in shared memory                11.32 ms    7.51 ms
+//   this layout                                               8.35       4.69
+//   constants instead of tables                               8.04       4.53
+//   one thread per transform line, straight from the rows     7.92       4.36
+//   A-terms two pixels ahead                                  7.93       4.15
+// The tensor pipe is 50 % busy (16 cycles per visibility at full rate), issue slots 47 %: a
+// CTA's chain per tile (A 1250, MMAs 2 x 1024, sums 2 x 500 cycles, measured alone) leaves
+// the tensor cores to the other CTA for just over half its length, and tensor memory has no
+// room for a second A beside the accumulator.  Short subgrids are bound by the prologue
+// (8 k of 12 k cycles).  Measured and not kept: a coefficient warp (8.53 ms: the
+// coefficients were already hidden), MMAs issued by a worker (9.2: issuing blocks the
+// warp), A's first half formed during the sums (spills: + 25 %).
 // Every wait is bounded; after a failed wait a thread skips every later wait,
 // the error word is set and no output is written.
 #include "batch_jobs.cuh"

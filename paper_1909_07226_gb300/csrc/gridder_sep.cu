@@ -25,36 +25,54 @@
 // two with max |c_k| sigma <= 1.
 //
 // Precision.  Both operands are split into FP16 hi + lo parts (A after a
-// power-of-two scale per subgrid).  The m = 0 block takes A_hi B_hi +
-// A_hi B_lo + A_lo B_hi; the m = 1 block, which contributes at most theta
-// relative, takes A_hi B_hi only.  One MMA of N = 192 computes
-// A_hi [B_hi (128 rows) | B_lo (m = 0, 64 rows)], a second of N = 64 adds
+// power-of-two scale per subgrid), hi a multiple of a fixed quantum that FP16
+// holds exactly, so that hi + lo is exact up to the rounding of lo.  The m = 0
+// block takes A_hi B_hi + A_hi B_lo + A_lo B_hi; the m = 1 block, which
+// contributes at most theta relative, takes A_hi B_hi only.  One MMA of N = 192
+// computes A_hi [B_hi (128 rows) | B_lo (m = 0, 64 rows)], a second of N = 64 adds
 // A_lo B_hi (m = 0) to the correction columns.  The tensor cores accumulate
-// without rounding to nearest, so every FOLD groups of 8 visibilities the
-// accumulator is added into FP32 sums in shared memory (RN) and restarted.
-// The producers read it as soon as the period's MMAs are done and release it
-// before adding, so the MMAs wait only for the tensor-memory loads; the rest
-// of the tensor memory holds two A stages.
+// without rounding to nearest, so every 512 visibilities the accumulator is folded
+// into the FP32 image in shared memory (RN) and restarted; the fold applies
+// I = S0 + i r S1 / sigma, so it keeps one complex image, half of S0 and S1.
 //
-// Schedule.  One CTA per subgrid, one CTA per SM: sixteen producer warps and
-// one MMA warp.  A stage is eight groups of 8 visibilities: every stage ends
-// in a tensor-memory wait, a proxy fence and a barrier arrival per warp, and
-// with eight groups (rather than four) that fixed cost is spread over twice
-// the work, 9 % off the gridder's time.  Per stage each producer, for each of
-// its groups warp / 4 and warp / 4 + 4:
-//   - writes the 8 A entries of its row (polarisation lane / 8, pixel row
-//     8 (warp % 4) + lane % 8) into tensor memory, one 16-column store.  It
-//     forms Ey for two of the visibilities and takes the others from the
-//     lanes of the same row by shuffles;
-//   - forms the B entries of pixel column 8 (warp % 4) + lane % 8 for the
-//     adjacent visibilities 2 (lane / 8) and 2 (lane / 8) + 1 of the group,
-//     and writes them as one 8-byte store per row block (a warp's store
-//     covers 256 contiguous bytes, free of bank conflicts).
-// Visibilities are staged 512 at a time; the next batch is loaded into
-// registers while the current one is processed.
-// Tensor memory (512 columns):
+// Schedule.  One CTA per subgrid and two CTAs per SM (half the tensor memory and 106
+// of 227 KB shared memory each): one CTA's start, folds, transform and adder run under
+// the other's sums.  A CTA has two sets of four producer warps, an MMA warp and a
+// loader warp.  The sets take turns: a stage is two groups of 8 visibilities of one
+// set.  Per group, warp yq of the set
+//   - forms A of the 8 pixel rows y = 8 yq .. + 7 and all four polarisations (its
+//     lane quarter of tensor memory).  The 16 x 256-bit store form gives a thread
+//     four of the quarter's rows for two visibilities: two pixel rows x two
+//     polarisations, so that each Ey and each V is used twice, without shuffles;
+//   - forms B of the pixel columns x = 8 yq .. + 7 (at L = 24 and 16 the quarters
+//     without A rows take the B blocks).
+// A and B of a group are formed side by side (their chains of phase, sine and cosine,
+// split and conversion overlap); A's stage buffer is freed by the set's previous
+// MMAs, B has two buffers per set.  Visibilities are staged 256 at a time, as pairs:
+// the first batch by the producers, the others by the loader warp, which keeps their
+// loads out of the producers' registers.
+// Tensor memory (256 columns):
 //   accumulator: main (m, re/im, x) 0..127, correction (m = 0) 128..191
-//   A stage s at 192 + 128 s, group i at + 16 i: 8 columns hi, 8 lo
+//   A of set s at 192 + 32 s, group i at + 16 i: 8 columns hi, 8 lo
+//
+// What bounds it, and what the choices measured (LOFAR-like plan, 73.9 M visibilities in
+// 45.9 k subgrids of about 1600; and the same array with A-terms every 16 s, 18.4 M in
+// 89.4 k of about 206):
+//   one CTA per SM, 16 producer warps, Ey by shuffles        13.42 ms    7.65 ms
+//   two CTAs, fragment stores, exact hi/lo split             13.03       5.62
+//   one thread per transform line, columns straight to the
+//   grid (the pixel passes around the transform cost a
+//   third of a short subgrid's instructions)                 12.69       5.09
+//   B around the A stores, A and B side by side              12.02       4.88
+//   loader warp (short subgrids: no gain)                    11.51       4.98
+//   A-terms ahead in registers instead of late bulk copies   11.43       4.82
+//   two rows x two polarisations per thread                  11.28       4.73
+// It is bound by latency and issue of the producers together: issue slots 54 %, the
+// shared-memory data pipe 60 %, the tensor pipe 35 % busy; leaving out any one of the
+// V loads, the split, the phasors or the MMA width gains 1 to 10 %.  Measured and not
+// kept: one group per stage with two buffers (a stage's hand-over costs each warp
+// about 670 cycles: 15.7 ms), polling by the producers (13.2), eight columns per fold
+// step (1.46 against 1.42 Mcycles on the first 256 timesteps).
 // Every wait is bounded; after a failed wait a thread skips every later wait,
 // the error word is set and no output is written.
 #include "batch_jobs.cuh"
@@ -84,9 +102,9 @@ constexpr int SPB = VB / (8 * SG);             // stages per batch
 constexpr int SPP = 2 * SPB;                   // stages per accumulation period (512 visibilities)
 constexpr uint32_t TMEM_COLS = 256;            // two CTAs share an SM's 512
 
-// Layout for subgrid size L (32, 24 or 16).  A has 128 rows: lane quarter yq holds pixel
-// rows y = 8 yq + ylo at lanes 8 q + ylo (quarters from L / 8 on are not used: their rows of
-// the accumulator are never read).  B has 6 L rows per group: (m = 0, re), (m = 0, im),
+// Layout for subgrid size L (32, 24 or 16).  A has 128 rows: lane quarter yq holds the pixel
+// rows y = 8 yq .. + 7 of the four polarisations (see the A entries; quarters from L / 8 on are
+// not used: their rows of the accumulator are never read).  B has 6 L rows per group: (m = 0, re), (m = 0, im),
 // (m = 1, re), (m = 1, im), then the lo parts of m = 0 re and im, L rows each.
 template <int L>
 struct SepG {
@@ -401,8 +419,10 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
             }
         };
 
-        // A entries: lane = 4 ylo + jp forms Ey of row y = 8 yq + ylo for visibilities 2 jp and 2 jp + 1
-        // of a group and multiplies the four polarisations with it (16 x 256-bit fragments)
+        // A entries of a group: row 8 a + b of the quarter is polarisation 2 (b / 4) + a / 2, pixel row
+        // y = 8 yq + 4 (a % 2) + b % 4; lane 4 b + jp holds rows b, 8 + b, 16 + b and 24 + b of the
+        // visibilities 2 jp and 2 jp + 1 (the 16 x 256-bit fragments), so it forms Ey for two y and
+        // multiplies two polarisations with each
         const int jp = lane & 3, qh = lane >> 4;
         const int y0 = 8 * yq + ((lane >> 2) & 3);
         const float Yv = (float)(y0 - SL / 2);

@@ -47,13 +47,6 @@ __device__ __forceinline__ void mma_ta_i(uint32_t dtmem, uint32_t atmem, uint64_
                  :: "r"(dtmem), "r"(atmem), "l"(db), "r"(idesc), "r"(acc) : "memory");
 }
 
-// D (tensor memory) += A (shared memory, 128 x 16 K-major) x B (shared memory, N x 16 K-major)^T
-__device__ __forceinline__ void mma_ss_i(uint32_t dtmem, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
-    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
-                 " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-                 :: "r"(dtmem), "l"(da), "l"(db), "r"(idesc), "r"(acc) : "memory");
-}
-
 // D (tensor memory) += A (tensor memory, 128 x 16) x B (shared memory, 16 x 16)^T; acc = 0 overwrites
 __device__ __forceinline__ void mma_ta(uint32_t dtmem, uint32_t atmem, uint64_t db, uint32_t acc) {
     asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
@@ -172,10 +165,6 @@ __device__ __forceinline__ void tmem_st(uint32_t taddr, const uint32_t (&v)[4]) 
                  :: "r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
 }
 
-__device__ __forceinline__ void tmem_st2(uint32_t taddr, uint32_t v0, uint32_t v1) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};" :: "r"(taddr), "r"(v0), "r"(v1) : "memory");
-}
-
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16]) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
                  :: "r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]),
@@ -226,20 +215,6 @@ __device__ __forceinline__ void split_e(float x, float y, uint32_t &hi, uint32_t
         " fma.rn.f32.f16 ly, hy, m1, %3;\n"
         " cvt.rn.f16x2.f32 %1, ly, lx;\n"
         "}" : "=r"(hi), "=r"(lo) : "f"(x), "f"(y));
-}
-
-// split_e with the FP16 constant -1 (0xBC00) passed in a register that the
-// caller keeps live across its loop
-__device__ __forceinline__ void split_e_m(float x, float y, uint16_t m1, uint32_t &hi, uint32_t &lo) {
-    asm("{\n"
-        " .reg .b16 hx, hy;\n"
-        " .reg .f32 lx, ly;\n"
-        " cvt.rn.f16x2.f32 %0, %3, %2;\n"
-        " mov.b32 {hx, hy}, %0;\n"
-        " fma.rn.f32.f16 lx, hx, %4, %2;\n"
-        " fma.rn.f32.f16 ly, hy, %4, %3;\n"
-        " cvt.rn.f16x2.f32 %1, ly, lx;\n"
-        "}" : "=r"(hi), "=r"(lo) : "f"(x), "f"(y), "h"(m1));
 }
 
 // Programmatic dependent launch.  A kernel that calls allow_dependents() lets the next
