@@ -45,10 +45,10 @@ LANES_PER_SM = 128
 ISSUE_PER_VISPIX_TC = 9
 # DRAM bytes (read + write) per visibility-pixel of one launch, from the ncu
 # capture of the separable kernels (the default at L = 32 where the plan is
-# separable) on the LOFAR-like slice, one launch of all 3206 subgrids, 4.731e9
-# visibility-pixels: gridder 178.3 + 5.7 MB (visibilities and coordinates in; the
+# separable) on the LOFAR-like slice, one launch of all its subgrids, 4.731e9
+# visibility-pixels: gridder 178.5 MB (visibilities and coordinates in; the
 # atomically updated grid lines are still dirty in L2 when the launch ends), degridder
-# 31.1 + 92.4 MB
+# 120.8 MB
 # (grid lines and coordinates in, model visibilities out).  The traffic is
 # proportional to the work, so it scales to a full launch by the units processed.
 # Kernels without a capture of their current code report no traffic.
@@ -77,8 +77,8 @@ DTYPE_SEP = "f32 (fp16 hi/lo split tensor-core products, fp32 accumulate)"
 DTYPE_MIXED = ("f32 (fp16 hi/lo split tensor-core products for subgrids within the separable bound and "
                "pieces, packed fp32 for the rest; fp32 accumulate)")
 KERNEL_TRAFFIC = {
-    "gridder": {SEP_VARIANT: (178.5e6 + 5.6e6) / 4.731e9},
-    "degridder": {SEP_VARIANT: (31.2e6 + 92.4e6) / 4.731e9},
+    "gridder": {SEP_VARIANT: 178.5e6 / 4.731e9},
+    "degridder": {SEP_VARIANT: 120.8e6 / 4.731e9},
 }
 
 
