@@ -46,7 +46,7 @@
 //   constants instead of tables                               8.04       4.53
 //   one thread per transform line, straight from the rows     7.92       4.36
 //   A-terms two pixels ahead                                  7.93       4.15
-// The tensor pipe is 50 % busy (16 cycles per visibility at full rate), issue slots 47 %: a
+// The tensor pipe is 50 % busy (16 cycles per visibility at full rate), issue slots 46 %: a
 // CTA's chain per tile (A 1250, MMAs 2 x 1024, sums 2 x 500 cycles, measured alone) leaves
 // the tensor cores to the other CTA for just over half its length, and tensor memory has no
 // room for a second A beside the accumulator.  Short subgrids are bound by the prologue

@@ -67,8 +67,8 @@
 //   loader warp (short subgrids: no gain)                    11.51       4.98
 //   A-terms ahead in registers instead of late bulk copies   11.43       4.82
 //   two rows x two polarisations per thread                  11.28       4.73
-// It is bound by latency and issue of the producers together: issue slots 54 %, the
-// shared-memory data pipe 60 %, the tensor pipe 35 % busy; leaving out any one of the
+// It is bound by latency and issue of the producers together: issue slots 56 %, the
+// shared-memory data pipe 52 %, the tensor pipe 35 % busy; leaving out any one of the
 // V loads, the split, the phasors or the MMA width gains 1 to 10 %.  Measured and not
 // kept: one group per stage with two buffers (a stage's hand-over costs each warp
 // about 670 cycles: 15.7 ms), polling by the producers (13.2), eight columns per fold
