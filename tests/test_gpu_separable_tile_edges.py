@@ -57,3 +57,22 @@ def test_sizes_around_the_kernels_units(L, n_chan, n_t):
     assert launches == {"gridder": 1, "degridder": 1}        # fused, the separable kernels
     parity(g.cpu().numpy(), O.grid(wl, op), f"grid L={L} K={n_chan * n_t}")
     parity(v.cpu().numpy(), O.degrid(wl, op, G), f"degrid L={L} K={n_chan * n_t}")
+
+
+@pytest.mark.parametrize("L", [32, 24, 16])
+def test_degrid_into_an_8_byte_aligned_buffer(L):
+    # the fused separable degridder writes two polarisations at a time; a complex64 buffer
+    # may start at any multiple of 8 bytes
+    import torch
+    wl = syn.make_small(seed=260, n_st=3, n_t=40, n_chan=5, L=L, N=8 * L, max_t=40, n_slots=1, flag_p=0.1,
+                        diameter_m=100.0, cell=2.0e-4, df=0.2e6, dt=1.0)
+    p = idg.plan_from_workload(wl)
+    op = O.plan(wl)
+    assert p.stats.separable == 1 and p.stats.n_vis_dropped == 0 and op.desc[:, O.D_KP].min() >= 64
+    d = workload_to_device(wl)
+    G = syn.random_grid(np.random.default_rng(43), p.n_w_layers, wl.grid_size)
+    v = torch.full((wl.n_vis * 4 + 1,), complex(3.0, -7.0), dtype=torch.complex64, device="cuda")[1:].view(wl.vis.shape)
+    assert v.data_ptr() % 16 == 8
+    idg.degrid(p, dev(G), d["flags"], d["aterms"], d["taper"], v)
+    idg.device_errors()
+    parity(v.cpu().numpy(), O.degrid(wl, op, G), f"degrid L={L} into an 8-byte aligned buffer")
