@@ -50,7 +50,7 @@
 // split and conversion overlap); A's stage buffer is freed by the set's previous
 // MMAs, B has two buffers per set.  Visibilities are staged 256 at a time, as pairs:
 // the first batch by the producers, the others by the loader warp, which keeps their
-// loads out of the producers' registers.
+// loads out of the producers' registers; staging.h has the rules of the hand-over.
 // Tensor memory (256 columns):
 //   accumulator: main (m, re/im, x) 0..127, correction (m = 0) 128..191
 //   A of set s at 192 + 32 s, group i at + 16 i: 8 columns hi, 8 lo
@@ -78,6 +78,7 @@
 #include "batch_jobs.cuh"
 #include "device_common.cuh"
 #include "fft_impl.cuh"
+#include "staging.h"
 #include "tc_common.cuh"
 
 namespace idg {
@@ -156,7 +157,7 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
     float *s_vis = (float *)(smem + C::VIS_OFF);
     __shared__ uint32_t s_tmem;
     __shared__ __align__(8) uint64_t s_full[2], s_empty[2], s_foldbar, s_folded, s_drain,
-        s_staged, s_unstaged;
+        s_staged[kStagingBarriers], s_unstaged[kStagingBarriers];
     __shared__ float s_red[NPW];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -283,8 +284,10 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
         mbar_init(smem_u32(&s_foldbar), 1);
         mbar_init(smem_u32(&s_folded), NPW);
         mbar_init(smem_u32(&s_drain), 1);
-        mbar_init(smem_u32(&s_staged), 1);
-        mbar_init(smem_u32(&s_unstaged), NPW);
+        for (int k = 0; k < kStagingBarriers; ++k) {
+            mbar_init(smem_u32(&s_staged[k]), 1);
+            mbar_init(smem_u32(&s_unstaged[k]), NPW);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -349,16 +352,17 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
         at.step(32);
         if (n_batches > 1) load(raw, VB + lane < kp, at.t, at.c);
         for (int b = 1; b < n_batches; ++b) {
-            if (b >= 2) wait_or_fail(smem_u32(&s_unstaged), (uint32_t)(b & 1), failed);
+            const int bb = staging_buffer(b), bar = staging_barrier(b);
+            if (b >= kStagingBuffers) wait_or_fail(smem_u32(&s_unstaged[bar]), staging_free_parity(b), failed);
 #pragma unroll 1
             for (int i = lane; i < VB; i += 32) {
                 const Raw r = raw;
                 at.advance();
                 load(raw, b * VB + i + 32 < kp, at.t, at.c);
-                stage(r, scale, b & 1, i);
+                stage(r, scale, bb, i);
             }
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&s_staged));
+            if (lane == 0) mbar_arrive(smem_u32(&s_staged[bar]));
         }
         if (failed && lane == 0) atomicExch(&g_sep_error, 1);
     } else {
@@ -500,8 +504,8 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
         producers_sync();
         int next_fold = 0;
         for (int b = 0; b < n_batches; ++b) {
-            const int bb = b & 1;
-            if (b > 0) wait_or_fail(smem_u32(&s_staged), (uint32_t)((b - 1) & 1), failed);
+            const int bb = staging_buffer(b), bar = staging_barrier(b);
+            if (b > 0) wait_or_fail(smem_u32(&s_staged[bar]), staging_full_parity(b), failed);
             const float *cb = s_cb + bb * VB * 2, *ca = s_ca + bb * VB * 2, *vb = s_vis + bb * VB * 8;
             const int st_end = min((b + 1) * SPB, n_stages);
             // B of the stage's first (half 0) or second group (half 1); at L = 24 quarter 3 does the first
@@ -555,7 +559,7 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
                 }
             }
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&s_unstaged));
+            if (lane == 0) mbar_arrive(smem_u32(&s_unstaged[bar]));
         }
 #pragma unroll
         for (int ip = 0; ip < AHEAD; ++ip) load_aterms(ip);
