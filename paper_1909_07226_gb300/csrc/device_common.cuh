@@ -176,7 +176,8 @@ __device__ __forceinline__ f2_t f2_mul(f2_t a, f2_t b) {
 __device__ __forceinline__ f2_t f2_bcast(float v) { return f2_pack(v, v); }
 // v = hi + lo with hi the multiple of ulp(magic) nearest to v (magic = 1.5 x a power of two far
 // above |v|): exact.  For |v| <= 2048 ulp(magic), hi fits FP16 exactly, and lo, at most half
-// that ulp, is rounded by its own FP16 conversion at 2^-12 of itself.
+// that ulp, is rounded by its own FP16 conversion at 2^-12 of itself: an absolute error of 2^-13
+// ulp(magic), whatever the size of v.  For phasors, whose error counts against 1.
 __device__ __forceinline__ void f2_split(f2_t v, float magic, f2_t &hi, f2_t &lo) {
     hi = f2_add(f2_add(v, f2_bcast(magic)), f2_bcast(-magic));
     lo = f2_fma(hi, f2_bcast(-1.0f), v);

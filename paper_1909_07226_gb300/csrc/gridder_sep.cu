@@ -24,9 +24,13 @@
 // K = (k, r), so D[(q, y)][(m, x, re/im)] = (Re, Im) S_mq.  sigma is a power of
 // two with max |c_k| sigma <= 1.
 //
-// Precision.  Both operands are split into FP16 hi + lo parts (A after a
-// power-of-two scale per subgrid), hi a multiple of a fixed quantum that FP16
-// holds exactly, so that hi + lo is exact up to the rounding of lo.  The m = 0
+// Precision.  Both operands are split into FP16 hi + lo parts, A after a power-of-two scale per
+// subgrid, and hi + lo holds every value of A to 2^-22 of itself or 2^-13 of a quantum Q, whichever
+// is larger: hi is the FP16 value rounded to a multiple of Q, 2^-7 of its polarisation's geometric
+// mean |Re V| + |Im V| in the subgrid.  Without that rounding the tensor cores, which truncate, lose
+// the products' last bits at every step (1.4e-6 instead of 0.8e-6 of a grid); with one Q per
+// subgrid, below its largest value, a cross hand of 1 % would keep 11 bits (3e-5 of its grid).  B's
+// phasors are split at multiples of 2^-11: hi + lo holds them to 2^-24 of 1.  The m = 0
 // block takes A_hi B_hi + A_hi B_lo + A_lo B_hi; the m = 1 block, which
 // contributes at most theta relative, takes A_hi B_hi only.  One MMA of N = 192
 // computes A_hi [B_hi (128 rows) | B_lo (m = 0, 64 rows)], a second of N = 64 adds
@@ -67,10 +71,13 @@
 //   loader warp (short subgrids: no gain)                    11.51       4.98
 //   A-terms ahead in registers instead of late bulk copies   11.43       4.82
 //   two rows x two polarisations per thread                  11.28       4.73
+//   A's hi by its own size, rounded per polarisation (the
+//   figures above: one quantum per subgrid)                  11.41       4.84
 // It is bound by latency and issue of the producers together: issue slots 56 %, the
 // shared-memory data pipe 52 %, the tensor pipe 35 % busy; leaving out any one of the
 // V loads, the split, the phasors or the MMA width gains 1 to 10 %.  Measured and not
-// kept: one group per stage with two buffers (a stage's hand-over costs each warp
+// kept: A's hi rounded in FP32 with float means (11.72 and 4.94 ms: more registers, and the sums'
+// shuffles weigh on short subgrids); one group per stage with two buffers (a stage's hand-over costs each warp
 // about 670 cycles: 15.7 ms), polling by the producers (13.2), eight columns per fold
 // step (1.46 against 1.42 Mcycles on the first 256 timesteps).
 // Every wait is bounded; after a failed wait a thread skips every later wait,
@@ -159,6 +166,8 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
     __shared__ __align__(8) uint64_t s_full[2], s_empty[2], s_foldbar, s_folded, s_drain,
         s_staged[kStagingBarriers], s_unstaged[kStagingBarriers];
     __shared__ float s_red[NPW];
+    __shared__ int s_exp[NPW][5];
+    __shared__ __align__(8) uint32_t s_round[4];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool mma_warp = warp == MMA_WARP, producer = warp < NPW;
@@ -220,14 +229,14 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
         v[6 * VB] = b.z;
         v[6 * VB + 2] = b.w;
     };
-    // the subgrid's power-of-two scale: largest unflagged |component| of V in [2^9, 2^10)
+    // the subgrid's power-of-two scale: largest unflagged |component| of V in [2^11, 2^12)
     auto scale_exponent = [&]() {
         float m = 0.0f;
 #pragma unroll
         for (int w = 0; w < NPW; ++w) m = fmaxf(m, s_red[w]);
         int e2 = 0;
         if (m > 0.0f) frexpf(m, &e2);
-        return 10 - e2;
+        return min(12 - e2, 126);      // (a finite scale for the smallest inputs)
     };
     // timestep and channel (in the subgrid) of visibility k; advance() goes n visibilities on
     struct Where {
@@ -260,21 +269,43 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
         // read here once more, for the scale; they come back from L2 when they are staged)
         Where at(tid, d.nc);
         load(raw, tid < kp, at.t, at.c);
+        // and, per polarisation, the sum of the binary exponents of |Re| + |Im|
         float m = 0.0f;
+        int ex[4] = {}, n = 0;
+        auto add_exponents = [&](const float4 &a, const float4 &b) {
+            ex[0] += __float_as_int(fabsf(a.x) + fabsf(a.y)) >> 23;
+            ex[1] += __float_as_int(fabsf(a.z) + fabsf(a.w)) >> 23;
+            ex[2] += __float_as_int(fabsf(b.x) + fabsf(b.y)) >> 23;
+            ex[3] += __float_as_int(fabsf(b.z) + fabsf(b.w)) >> 23;
+            ++n;
+        };
         if (kp > VB) {
             at.step(VB);
 #pragma unroll 4
             for (int k = VB + tid; k < kp; k += VB) {
                 at.advance();
                 const size_t vi = (bt0 + at.t) * g.n_chan + d.c0 + at.c;
-                const float mk = max_of(vis[2 * vi], vis[2 * vi + 1]);
-                if (!(flags && flags[vi])) m = fmaxf(m, mk);
+                const float4 va = vis[2 * vi], vb = vis[2 * vi + 1];
+                if (!(flags && flags[vi])) {
+                    m = fmaxf(m, max_of(va, vb));
+                    add_exponents(va, vb);
+                }
             }
         }
-        if (raw.in && !raw.flag) m = fmaxf(m, max_of(raw.a, raw.b));
+        if (raw.in && !raw.flag) {
+            m = fmaxf(m, max_of(raw.a, raw.b));
+            add_exponents(raw.a, raw.b);
+        }
+        m = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m)));      // (m >= 0)
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-        if (lane == 0) s_red[warp] = m;
+        for (int q = 0; q < 4; ++q) ex[q] = __reduce_add_sync(0xffffffffu, ex[q]);
+        n = __reduce_add_sync(0xffffffffu, n);
+        if (lane == 0) {
+            s_red[warp] = m;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) s_exp[warp][q] = ex[q];
+            s_exp[warp][4] = n;
+        }
     }
     if (tid == 0) {
         for (int s = 0; s < 2; ++s) {
@@ -370,9 +401,7 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
         const float scale = ldexpf(1.0f, ex), inv_scale = ldexpf(1.0f, -ex);
         const uint32_t lane_base = tmem + ((uint32_t)(32 * yq) << 16);
         const float csig = g.c_scale, rs = 1.0f / csig;
-        // FP16 hi/lo split points: A's |components| are below 2^10 sqrt(2) (integers fit FP16 up to
-        // 2^11), B's at most 1 (multiples of 2^-11)
-        constexpr float magic_a = 12582912.0f, magic_1 = 6144.0f;
+        constexpr float magic_1 = 6144.0f;      // B's hi: multiples of 2^-11
 
         // one period's accumulator, I = S0 + i r S1 / sigma of this thread's row (polarisation
         // lane / 8, y = 8 yq + lane % 8) and its set's x, added to the image in FP32 (RN); the
@@ -432,7 +461,7 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
         const float Yv = (float)(y0 - SL / 2);
         const f2_t Y2[2] = {f2_bcast(Yv), f2_bcast(Yv + 4.0f)};
         const f2_t ty2[2] = {f2_bcast(yq < NQ ? g.sep[SL + y0] : 0.0f), f2_bcast(yq < NQ ? g.sep[SL + y0 + 4] : 0.0f)};
-        auto a_unit = [&](const float *cb, const float *vb, int pair, uint32_t (&e)[16]) {
+        auto a_unit = [&](const float *cb, const float *vb, int pair, const uint32_t (&round_a)[2], uint32_t (&e)[16]) {
             const ulonglong2 cf = *(const ulonglong2 *)(cb + 4 * (pair + jp));
             f2_t c2[2], s2[2], n2[2];
 #pragma unroll
@@ -450,12 +479,9 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
                 const ulonglong2 v = *(const ulonglong2 *)(vb + 2 * VB * (2 * qh + ql) + 4 * (pair + jp));
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    f2_t hr, lr, hi, li;
-                    f2_split(f2_fma(v.y, n2[h], f2_mul(v.x, c2[h])), magic_a, hr, lr);
-                    f2_split(f2_fma(v.y, c2[h], f2_mul(v.x, s2[h])), magic_a, hi, li);
                     const int k = 8 * ql + 2 * h;
-                    pack_pairs(hr, hi, e[k], e[k + 1]);
-                    pack_pairs(lr, li, e[k + 4], e[k + 5]);
+                    split_pairs(f2_fma(v.y, n2[h], f2_mul(v.x, c2[h])), f2_fma(v.y, c2[h], f2_mul(v.x, s2[h])),
+                                round_a[ql], e[k], e[k + 1], e[k + 4], e[k + 5]);
                 }
             }
         };
@@ -501,7 +527,22 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
         x_pair(xown, X2, sx2);
 
         stage(raw, scale, 0, tid);
+        // the quantum Q of A's hi per polarisation: 2^-7 of the geometric mean of |Re V| + |Im V|, as
+        // 1536 Q in FP16 (a number with that ulp); 0 (no rounding to it) where there is nothing to go by
+        if (warp == 0 && lane < 4) {
+            int sum = 0, n = 0;
+#pragma unroll
+            for (int w = 0; w < NPW; ++w) {
+                sum += s_exp[w][lane];
+                n += s_exp[w][4];
+            }
+            const int e = n > 0 ? sum / n - 127 + ex - 7 : -127;
+            const float r = e >= -24 && e <= 5 ? ldexpf(1536.0f, e) : 0.0f;
+            s_round[lane] = pack_f16x2(r, r);
+        }
         producers_sync();
+        const uint2 r2 = *(const uint2 *)(s_round + 2 * qh);
+        const uint32_t round_a[2] = {r2.x, r2.y};
         int next_fold = 0;
         for (int b = 0; b < n_batches; ++b) {
             const int bb = staging_buffer(b), bar = staging_barrier(b);
@@ -533,7 +574,7 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
                 // A and B of a group side by side, so that their chains (phase, sine and cosine, split)
                 // overlap.  The B buffer's last reader was the stage before the one waited for here
                 uint32_t e[16];
-                if (yq < NQ) a_unit(cb, vb, pair, e);
+                if (yq < NQ) a_unit(cb, vb, pair, round_a, e);
                 b_half(pair, Bs, 0);
                 if (use > 0) {       // the MMAs of the set's previous stage are done with A
                     wait_or_fail(smem_u32(&s_empty[set]), (uint32_t)((use - 1) & 1), failed);
@@ -542,7 +583,7 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
                 if (yq < NQ) {
                     tmem_st_16x256b(ta, e);
                     tmem_st_16x256b(ta + (16u << 16), e + 8);
-                    a_unit(cb, vb, pair + 4, e);
+                    a_unit(cb, vb, pair + 4, round_a, e);
                     tmem_st_16x256b(ta + 16u, e);
                     tmem_st_16x256b(ta + 16u + (16u << 16), e + 8);
                 }

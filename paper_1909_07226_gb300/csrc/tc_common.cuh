@@ -9,6 +9,8 @@
 
 #include <cstdint>
 
+#include "device_common.cuh"
+
 namespace idg {
 namespace tc {
 
@@ -201,6 +203,29 @@ __device__ __forceinline__ void pack_pairs(unsigned long long x, unsigned long l
     w1 = pack_f16x2(x1, y1);
 }
 
+// FP16 pair h rounded to a multiple of ulp(r) (r = 1.5 x a power of two; 0: h)
+__device__ __forceinline__ uint32_t round_f16x2(uint32_t h, uint32_t r) {
+    uint32_t v;
+    asm("{\n .reg .b32 t;\n add.rn.f16x2 t, %1, %2;\n sub.rn.f16x2 %0, t, %2;\n}" : "=r"(v) : "r"(h), "r"(r));
+    return v;
+}
+
+// FP16 pair of (x, y) less the FP16 pair hi, the differences formed exactly (hi within a factor of
+// two of the value, or zero)
+__device__ __forceinline__ uint32_t rest_e(uint32_t hi, float x, float y) {
+    uint32_t lo;
+    asm("{\n"
+        " .reg .b16 hx, hy, m1;\n"
+        " .reg .f32 lx, ly;\n"
+        " mov.b16 m1, 0xBC00;\n"
+        " mov.b32 {hx, hy}, %1;\n"
+        " fma.rn.f32.f16 lx, hx, m1, %2;\n"
+        " fma.rn.f32.f16 ly, hy, m1, %3;\n"
+        " cvt.rn.f16x2.f32 %0, ly, lx;\n"
+        "}" : "=r"(lo) : "r"(hi), "f"(x), "f"(y));
+    return lo;
+}
+
 // FP16 hi/lo parts of (x, y): hi = fp16 rounded, lo = fp16(v - hi) with v - hi formed
 // exactly by one mixed-precision fma per component (FP16 hi times -1 plus FP32 v).
 // Low halves hold x.
@@ -215,6 +240,22 @@ __device__ __forceinline__ void split_e(float x, float y, uint32_t &hi, uint32_t
         " fma.rn.f32.f16 ly, hy, m1, %3;\n"
         " cvt.rn.f16x2.f32 %1, ly, lx;\n"
         "}" : "=r"(hi), "=r"(lo) : "f"(x), "f"(y));
+}
+
+// FP16 hi/lo parts of (x0, y0) and (x1, y1) for packed x and y: hi the FP16 value rounded to a multiple
+// of a quantum Q, round = 1536 Q in both halves (0: not rounded further), lo = fp16(v - hi) with v - hi
+// exact.  hi is a multiple of Q or, from 512 Q on, of FP16's own ulp or twice that: hi + lo holds v
+// to 2^-22 of itself or 2^-13 Q, whichever is larger.
+__device__ __forceinline__ void split_pairs(dev::f2_t x, dev::f2_t y, uint32_t round, uint32_t &h0, uint32_t &h1,
+                                            uint32_t &l0, uint32_t &l1) {
+    float x0, x1, y0, y1;
+    pack_pairs(x, y, h0, h1);
+    h0 = round_f16x2(h0, round);
+    h1 = round_f16x2(h1, round);
+    dev::f2_unpack(x, x0, x1);
+    dev::f2_unpack(y, y0, y1);
+    l0 = rest_e(h0, x0, y0);
+    l1 = rest_e(h1, x1, y1);
 }
 
 // Programmatic dependent launch.  A kernel that calls allow_dependents() lets the next
