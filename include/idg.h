@@ -590,13 +590,25 @@ idg_status idg_device_errors(idg_stream stream);
  * Self-test of that failure path (no counterpart in the paper): enqueues on
  * `stream` one CTA that allocates tensor memory as the tensor-core kernels do,
  * waits on a shared-memory barrier that nothing arrives on, with a limit of
- * max_polls polls (1 .. 2^20, a few milliseconds at most), records the timeout
+ * max_polls polls (1 .. 2^20, 76 milliseconds at most), records the timeout
  * in its device error word and releases the tensor memory.  The next
  * idg_device_errors then returns IDG_ERR_TIMEOUT (and clears the word); the
  * device stays usable.  No matrix operation or copy is involved.
  * IDG_ERR_INVALID_ARG for max_polls out of range.
  */
 idg_status idg_selftest_wait_timeout(int64_t max_polls, idg_stream stream);
+
+/*
+ * The same for the separable tensor-core kernels: grids d_vis into d_grid and
+ * degrids d_model into d_vis_out (shapes as for idg_grid and idg_degrid; d_aterms may
+ * be NULL; no flags, the default taper) with the thread that issues a CTA's matrix
+ * operations giving up at its first wait, before it has issued any.  The next
+ * idg_device_errors returns IDG_ERR_TIMEOUT, and neither d_grid nor d_vis_out has
+ * been written.  IDG_ERR_UNSUPPORTED unless every subgrid of the plan takes those
+ * kernels.
+ */
+idg_status idg_selftest_issue_timeout(const idg_plan *plan, const void *d_vis, const void *d_model,
+                                      const void *d_aterms, void *d_grid, void *d_vis_out, idg_stream stream);
 
 /*
  * Anti-aliasing windows (Sect. 4.1-4.3 and the appendix; host, FP64, no GPU).

@@ -1624,6 +1624,26 @@ idg_status idg_grid_degrid_host(const idg_plan *p, const void *h_vis, const void
 }
 
 // ---------------------------------------------------------------------------
+// self-test of the separable kernels' failure path
+
+idg_status idg_selftest_issue_timeout(const idg_plan *p, const void *vis, const void *model, const void *aterms,
+                                      void *grid, void *vis_out, idg_stream stream) {
+    idg_status st = check_call(p, vis, "d_vis", grid, "d_grid");
+    if (st != IDG_OK) return st;
+    if (!model) return fail(IDG_ERR_INVALID_ARG, "d_model is NULL");
+    if (!vis_out) return fail(IDG_ERR_INVALID_ARG, "d_vis_out is NULL");
+    if (!p->stats.separable || !separable_size(p->L))
+        return fail(IDG_ERR_UNSUPPORTED, "the self-test needs L = 32, 24 or 16 and a separable plan");
+    const float *taper = p->taper_or_default(nullptr);
+    if (!taper) return no_default_taper();
+    const Geometry g = p->geometry();
+    const SubgridSet all = order_set(p, 0, p->stats.n_subgrids);
+    st = launch_gridder_sep_give_up(g, all, vis, aterms, taper, grid, stream);
+    if (st == IDG_OK) st = launch_degridder_sep_give_up(g, all, model, aterms, taper, vis_out, stream);
+    return st;
+}
+
+// ---------------------------------------------------------------------------
 // stage entry points
 
 idg_status idg_grid_subgrids(const idg_plan *p, int64_t first, int64_t count, const void *vis,

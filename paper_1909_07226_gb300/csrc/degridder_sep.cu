@@ -53,8 +53,9 @@
 // (8 k of 12 k cycles).  Measured and not kept: a coefficient warp (8.53 ms: the
 // coefficients were already hidden), MMAs issued by a worker (9.2: issuing blocks the
 // warp), A's first half formed during the sums (spills: + 25 %).
-// Every wait is bounded; after a failed wait a thread skips every later wait,
-// the error word is set and no output is written.
+// Every wait is bounded.  After one that runs out a thread skips every later wait, the MMA thread
+// issues no more MMAs, the error word is set and nothing is written any more (the visibilities of
+// the tiles before it have been).
 #include "batch_jobs.cuh"
 #include "device_common.cuh"
 #include "fft_impl.cuh"
@@ -173,7 +174,8 @@ __device__ __forceinline__ void form_ey(const Geometry &g, float cb, float cc, f
 // Visibilities of subgrid d of geometry g from its image src[L][L][4], or with
 // FUSED from the grid src[layer][N][N][4]: split and transformed in shared memory
 // first (Algorithm 2: split from the master grid, "IFFT", image-domain kernel, sum).
-template <int L, bool FUSED>
+// NEVER: the self-test's form, whose MMA thread gives up at once.
+template <int L, bool FUSED, bool NEVER = false>
 __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevSubgrid d,
                                                    const float4 *__restrict__ src, const uint8_t *__restrict__ flags,
                                                    const float4 *__restrict__ aterms, const float *__restrict__ taper,
@@ -184,6 +186,7 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
     float4 *s_part = (float4 *)(smem + C::PART_OFF);
     __shared__ uint32_t s_tmem;
     __shared__ __align__(8) uint64_t s_afull, s_dfull, s_dempty, s_drain, s_gbar;
+    __shared__ int s_given_up;
     __shared__ float s_red[NWW];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -198,6 +201,7 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
         // barriers by lane 0; then one bulk copy per lane: the subgrid's grid rows (32 L bytes
         // each, contiguous in the grid)
         if (lane == 0) {
+            s_given_up = 0;
             mbar_init(smem_u32(&s_afull), NWW);
             mbar_init(smem_u32(&s_dfull), 1);
             mbar_init(smem_u32(&s_dempty), NWW);
@@ -248,8 +252,7 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
     // ---- prologue: the corrected image P = taper A_p I A_q^H, this thread's pixels in registers
     if (FUSED) {
         bool late = false;
-        wait_or_fail(smem_u32(&s_gbar), 0u, late);
-        if (late) atomicExch(&g_sepd_error, 1);
+        wait_or_fail(smem_u32(&s_gbar), 0u, late, &s_given_up);
         // one thread per line and polarisation: columns from the grid rows, then rows into the image
         const int pol = tid & 3, ln = tid >> 2;
         const float2 *src_col = (const float2 *)smem + 4 * ln + pol;
@@ -357,11 +360,12 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
         if (lane == 0) {
             const uint64_t db0 = smem_desc(smem_u32(smem));
             const uint32_t at = tmem + C::A_COL;
-            for (int t = 0; t < n_tiles; ++t) {
-                poll_or_fail(smem_u32(&s_afull), (uint32_t)(t & 1), failed);
+            for (int t = 0; t < n_tiles && !failed; ++t) {
+                poll_or_fail<NEVER>(smem_u32(&s_afull), (uint32_t)(t & 1), failed, &s_given_up);
                 for (int p = 0; p < C::PARTS; ++p) {
                     const int n = t * C::PARTS + p;
-                    if (n > 0) poll_or_fail(smem_u32(&s_dempty), (uint32_t)((n - 1) & 1), failed);
+                    if (n > 0) poll_or_fail<NEVER>(smem_u32(&s_dempty), (uint32_t)((n - 1) & 1), failed, &s_given_up);
+                    if (failed) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint64_t dbp = db0 + (uint64_t)((p * C::PN * 32) >> 4);
 #pragma unroll
@@ -377,10 +381,8 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
                 }
             }
             commit(smem_u32(&s_drain));
-            bool drained = false;
-            wait_or_fail(smem_u32(&s_drain), 0u, drained);     // bounded: let own MMAs finish before the free
+            if (!mbar_wait(smem_u32(&s_drain), 0u)) s_given_up = 1;     // bounded: let own MMAs finish before the free
         }
-        failed = __shfl_sync(0xffffffffu, failed, 0);
     } else {
         const uint32_t lane_base = tmem + ((uint32_t)(32 * quarter) << 16);
         const float csig = g.c_scale;
@@ -403,8 +405,9 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
         uint32_t ovi = 0xFFFFFFFFu;
         auto finish = [&](int t) {
             pair_sync(quarter);
+            const bool lost = *(const volatile int *)&s_given_up;     // (also what the other half saw before)
             const float4 o = s_part[((t & 1) * 2 + half) * TV + row];
-            if (ovi != 0xFFFFFFFFu && !failed) {
+            if (ovi != 0xFFFFFFFFu && !lost) {
                 float4 v = make_float4((own.x + o.x) * inv_scale, (own.y + o.y) * inv_scale, (own.z + o.z) * inv_scale,
                                        (own.w + o.w) * inv_scale);
                 if (ovi & 0x80000000u) v = make_float4(0.f, 0.f, 0.f, 0.f);      // flagged
@@ -443,7 +446,7 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
                     form_coef(ca, cb, cc, vi);
                     load_raw((t + 2) * TV + row);
                 }
-                wait_or_fail(smem_u32(&s_dfull), (uint32_t)((t * C::PARTS + p) & 1), failed);
+                wait_or_fail(smem_u32(&s_dfull), (uint32_t)((t * C::PARTS + p) & 1), failed, &s_given_up);
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 if (active) {
                     // y_q = sum_y (cs - i sn) T_q(y): Re = sum cs Tr + sn Ti, Im = sum cs Ti - sn Tr
@@ -498,10 +501,10 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
             }
         }
         if (n_tiles > 0 && (n_tiles - 1) * TV + 32 * quarter < kp) finish(n_tiles - 1);
-        if (failed && lane == 0) atomicExch(&g_sepd_error, 1);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (tid == 0 && s_given_up) atomicExch(&g_sepd_error, 1);
     if (warp == MMA_WARP)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "n"(TMEM_COLS));
 }
@@ -526,6 +529,27 @@ degridder_sep_fused_kernel(Geometry g, const int32_t *__restrict__ idx, int64_t 
     const int sid = idx ? idx[blockIdx.x] : (int)(first + blockIdx.x);
     degridder_sep_body<L, true>(g, g.sub[sid], grid, flags, aterms, taper, vis_out);
     complete_after_primary();
+}
+
+// the fused kernel's self-test: see idg_selftest_issue_timeout
+template <int L>
+__global__ void __launch_bounds__(NT, CTAS)
+degridder_sep_give_up_kernel(Geometry g, const int32_t *__restrict__ idx, const float4 *__restrict__ grid,
+                             const float4 *__restrict__ aterms, const float *__restrict__ taper,
+                             float4 *__restrict__ vis_out) {
+    degridder_sep_body<L, true, true>(g, g.sub[idx[blockIdx.x]], grid, nullptr, aterms, taper, vis_out);
+}
+
+template <int L>
+idg_status launch_give_up(const Geometry &g, const SubgridSet &set, const void *grid, const void *aterms,
+                          const float *taper, void *vis_out, cudaStream_t s) {
+    auto kern = degridder_sep_give_up_kernel<L>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SepD<L>::SMEM);
+    if (e != cudaSuccess) return cuda_fail(e, "separable degridder smem attribute");
+    kern<<<(unsigned)set.count, NT, SepD<L>::SMEM, s>>>(g, set.idx, (const float4 *)grid, (const float4 *)aterms, taper,
+                                                       (float4 *)vis_out);
+    e = cudaGetLastError();
+    return e == cudaSuccess ? IDG_OK : cuda_fail(e, "separable degridder self-test launch");
 }
 
 template <int L>
@@ -598,6 +622,18 @@ idg_status launch_degridder_sep_fused(const Geometry &g, const SubgridSet &set, 
     case 32: return launch_sepd_set<32>(true, g, set, grid, flags, aterms, taper, vis_out, (cudaStream_t)stream);
     case 24: return launch_sepd_set<24>(true, g, set, grid, flags, aterms, taper, vis_out, (cudaStream_t)stream);
     default: return launch_sepd_set<16>(true, g, set, grid, flags, aterms, taper, vis_out, (cudaStream_t)stream);
+    }
+}
+
+idg_status launch_degridder_sep_give_up(const Geometry &g, const SubgridSet &set, const void *grid, const void *aterms,
+                                        const float *taper, void *vis_out, void *stream) {
+    if (!separable_size(g.L) || !g.separable || !set.idx)
+        return fail(IDG_ERR_UNSUPPORTED, "the separable degridder needs L = 32, 24 or 16 and a separable plan");
+    if (set.count <= 0) return IDG_OK;
+    switch (g.L) {
+    case 32: return launch_give_up<32>(g, set, grid, aterms, taper, vis_out, (cudaStream_t)stream);
+    case 24: return launch_give_up<24>(g, set, grid, aterms, taper, vis_out, (cudaStream_t)stream);
+    default: return launch_give_up<16>(g, set, grid, aterms, taper, vis_out, (cudaStream_t)stream);
     }
 }
 

@@ -80,8 +80,8 @@
 // shuffles weigh on short subgrids); one group per stage with two buffers (a stage's hand-over costs each warp
 // about 670 cycles: 15.7 ms), polling by the producers (13.2), eight columns per fold
 // step (1.46 against 1.42 Mcycles on the first 256 timesteps).
-// Every wait is bounded; after a failed wait a thread skips every later wait,
-// the error word is set and no output is written.
+// Every wait is bounded.  After one that runs out a thread skips every later wait, the MMA thread
+// issues no more MMAs, the error word is set and the subgrid is not written.
 #include "batch_jobs.cuh"
 #include "device_common.cuh"
 #include "fft_impl.cuh"
@@ -145,9 +145,10 @@ __device__ __forceinline__ void producers_sync() { asm volatile("bar.sync 1, %0;
 // in the same place, or the transforms added into the grid o[layer][N][N][4]
 enum Out { kImage, kTransform, kGrid };
 
+// NEVER: the self-test's form, whose MMA thread gives up at once.
 // One subgrid d of geometry g (Algorithm 1: direct sum, image-domain kernel, "FFT", add to the
 // master grid)
-template <int L, Out OUT>
+template <int L, Out OUT, bool NEVER = false>
 __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSubgrid d,
                                                  const float4 *__restrict__ vis, const uint8_t *__restrict__ flags,
                                                  const float4 *__restrict__ aterms, const float *__restrict__ taper,
@@ -165,6 +166,7 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
     __shared__ uint32_t s_tmem;
     __shared__ __align__(8) uint64_t s_full[2], s_empty[2], s_foldbar, s_folded, s_drain,
         s_staged[kStagingBarriers], s_unstaged[kStagingBarriers];
+    __shared__ int s_given_up;
     __shared__ float s_red[NPW];
     __shared__ int s_exp[NPW][5];
     __shared__ __align__(8) uint32_t s_round[4];
@@ -308,6 +310,7 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
         }
     }
     if (tid == 0) {
+        s_given_up = 0;
         for (int s = 0; s < 2; ++s) {
             mbar_init(smem_u32(&s_full[s]), NPW / 2);
             mbar_init(smem_u32(&s_empty[s]), 1);
@@ -351,9 +354,10 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
                 const int s = st & 1, use = st >> 1;        // set, and its how manieth stage
                 const bool first = st % SPP == 0, last = st % SPP == SPP - 1 || st == n_stages - 1;
                 if (first && st > 0) {         // the producers have read the previous period
-                    wait_or_fail(smem_u32(&s_folded), (uint32_t)(((st / SPP) - 1) & 1), failed);
+                    wait_or_fail(smem_u32(&s_folded), (uint32_t)(((st / SPP) - 1) & 1), failed, &s_given_up);
                 }
-                poll_or_fail(smem_u32(&s_full[s]), (uint32_t)(use & 1), failed);
+                poll_or_fail<NEVER>(smem_u32(&s_full[s]), (uint32_t)(use & 1), failed, &s_given_up);
+                if (failed) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const int ng = min(SG, total_groups - st * SG);
                 const uint64_t dbs = db0 + (uint64_t)(((2 * s + (use & 1)) * B_STAGE) >> 4);
@@ -370,11 +374,8 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
                 if (last) commit(smem_u32(&s_foldbar));
             }
             commit(smem_u32(&s_drain));
-            bool late = false;
-            wait_or_fail(smem_u32(&s_drain), 0u, late);     // bounded: let own MMAs finish before the free
-            if (late) failed = true;
+            if (!mbar_wait(smem_u32(&s_drain), 0u)) failed = true;     // bounded: let own MMAs finish before the free
         }
-        failed = __shfl_sync(0xffffffffu, failed, 0);
     } else if (warp == LOAD_WARP) {
         // batches 1 .. : 32 visibilities at a time, the next ones' loads in flight; a buffer is reused
         // once the producers are done with it
@@ -384,7 +385,7 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
         if (n_batches > 1) load(raw, VB + lane < kp, at.t, at.c);
         for (int b = 1; b < n_batches; ++b) {
             const int bb = staging_buffer(b), bar = staging_barrier(b);
-            if (b >= kStagingBuffers) wait_or_fail(smem_u32(&s_unstaged[bar]), staging_free_parity(b), failed);
+            if (b >= kStagingBuffers) wait_or_fail(smem_u32(&s_unstaged[bar]), staging_free_parity(b), failed, &s_given_up);
 #pragma unroll 1
             for (int i = lane; i < VB; i += 32) {
                 const Raw r = raw;
@@ -395,7 +396,6 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&s_staged[bar]));
         }
-        if (failed && lane == 0) atomicExch(&g_sep_error, 1);
     } else {
         const int ex = scale_exponent();
         const float scale = ldexpf(1.0f, ex), inv_scale = ldexpf(1.0f, -ex);
@@ -407,7 +407,7 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
         // lane / 8, y = 8 yq + lane % 8) and its set's x, added to the image in FP32 (RN); the
         // accumulator is released right after the loads
         auto fold = [&](int P) {
-            wait_or_fail(smem_u32(&s_foldbar), (uint32_t)(P & 1), failed);
+            wait_or_fail(smem_u32(&s_foldbar), (uint32_t)(P & 1), failed, &s_given_up);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             constexpr int XC = C::XC;
             if (yq < NQ) {
@@ -546,7 +546,7 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
         int next_fold = 0;
         for (int b = 0; b < n_batches; ++b) {
             const int bb = staging_buffer(b), bar = staging_barrier(b);
-            if (b > 0) wait_or_fail(smem_u32(&s_staged[bar]), staging_full_parity(b), failed);
+            if (b > 0) wait_or_fail(smem_u32(&s_staged[bar]), staging_full_parity(b), failed, &s_given_up);
             const float *cb = s_cb + bb * VB * 2, *ca = s_ca + bb * VB * 2, *vb = s_vis + bb * VB * 8;
             const int st_end = min((b + 1) * SPB, n_stages);
             // B of the stage's first (half 0) or second group (half 1); at L = 24 quarter 3 does the first
@@ -577,7 +577,7 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
                 if (yq < NQ) a_unit(cb, vb, pair, round_a, e);
                 b_half(pair, Bs, 0);
                 if (use > 0) {       // the MMAs of the set's previous stage are done with A
-                    wait_or_fail(smem_u32(&s_empty[set]), (uint32_t)((use - 1) & 1), failed);
+                    wait_or_fail(smem_u32(&s_empty[set]), (uint32_t)((use - 1) & 1), failed, &s_given_up);
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 }
                 if (yq < NQ) {
@@ -610,14 +610,15 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
         }
         if (n_periods == 0)
             for (int i = tid; i < 4 * FFT_S; i += NP) s_img[i] = make_float2(0.f, 0.f);
-        if (failed && lane == 0) atomicExch(&g_sep_error, 1);
     }
     // the taper of this thread's epilogue pixels
     float tw_pre[PIXT];
 #pragma unroll
     for (int i = 0; i < PIXT; ++i) tw_pre[i] = producer && tid + i * NP < SPIX ? taper[tid + i * NP] : 0.0f;
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    if (!__syncthreads_or(failed)) {
+    const bool lost = __syncthreads_or(failed);
+    if (lost && tid == 0) atomicExch(&g_sep_error, 1);
+    if (!lost) {
         // image-domain kernel per pixel: taper * A_p^H I A_q (with the centring factor when FUSED)
         if (producer) {
 #pragma unroll
@@ -700,6 +701,27 @@ gridder_sep_fused_kernel(Geometry g, const int32_t *__restrict__ idx, int64_t fi
     complete_after_primary();
 }
 
+// the fused kernel's self-test: see idg_selftest_issue_timeout
+template <int L>
+__global__ void __launch_bounds__(NT, CTAS)
+gridder_sep_give_up_kernel(Geometry g, const int32_t *__restrict__ idx, const float4 *__restrict__ vis,
+                           const float4 *__restrict__ aterms, const float *__restrict__ taper,
+                           float4 *__restrict__ grid) {
+    gridder_sep_body<L, kGrid, true>(g, g.sub[idx[blockIdx.x]], vis, nullptr, aterms, taper, grid);
+}
+
+template <int L>
+idg_status launch_give_up(const Geometry &g, const SubgridSet &set, const void *vis, const void *aterms,
+                          const float *taper, void *grid, cudaStream_t s) {
+    auto kern = gridder_sep_give_up_kernel<L>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SepG<L>::SMEM);
+    if (e != cudaSuccess) return cuda_fail(e, "separable gridder smem attribute");
+    kern<<<(unsigned)set.count, NT, SepG<L>::SMEM, s>>>(g, set.idx, (const float4 *)vis, (const float4 *)aterms, taper,
+                                                       (float4 *)grid);
+    e = cudaGetLastError();
+    return e == cudaSuccess ? IDG_OK : cuda_fail(e, "separable gridder self-test launch");
+}
+
 template <int L>
 idg_status launch_sep_set(Out out_kind, const Geometry &g, const SubgridSet &set, const void *vis, const uint8_t *flags,
                           const void *aterms, const float *taper, void *out, cudaStream_t s) {
@@ -774,6 +796,18 @@ idg_status launch_gridder_sep_transform(const Geometry &g, const SubgridSet &set
 idg_status launch_gridder_sep_fused(const Geometry &g, const SubgridSet &set, const void *vis, const uint8_t *flags,
                                     const void *aterms, const float *taper, void *grid, void *stream) {
     return launch_sep_any(kGrid, g, set, vis, flags, aterms, taper, grid, stream);
+}
+
+idg_status launch_gridder_sep_give_up(const Geometry &g, const SubgridSet &set, const void *vis, const void *aterms,
+                                      const float *taper, void *grid, void *stream) {
+    if (!separable_size(g.L) || !g.separable || !set.idx)
+        return fail(IDG_ERR_UNSUPPORTED, "the separable gridder needs L = 32, 24 or 16 and a separable plan");
+    if (set.count <= 0) return IDG_OK;
+    switch (g.L) {
+    case 32: return launch_give_up<32>(g, set, vis, aterms, taper, grid, (cudaStream_t)stream);
+    case 24: return launch_give_up<24>(g, set, vis, aterms, taper, grid, (cudaStream_t)stream);
+    default: return launch_give_up<16>(g, set, vis, aterms, taper, grid, (cudaStream_t)stream);
+    }
 }
 
 idg_status read_sep_error(int *code) {

@@ -255,6 +255,9 @@ idg_status launch_gridder_sep_transform(const Geometry &g, const SubgridSet &set
                                         const void *aterms, const float *taper, void *out, void *stream);
 idg_status launch_gridder_sep_fused(const Geometry &g, const SubgridSet &set, const void *vis, const uint8_t *flags,
                                     const void *aterms, const float *taper, void *grid, void *stream);
+// the self-test of its failure path: the same launch with MMA threads that give up at once
+idg_status launch_gridder_sep_give_up(const Geometry &g, const SubgridSet &set, const void *vis, const void *aterms,
+                                      const float *taper, void *grid, void *stream);
 idg_status read_sep_error(int *code);
 // separable tensor-core degridder (L = 32, 24 or 16, g.separable): from subgrid images, or
 // fused with the splitter and the inverse transform from grid
@@ -262,6 +265,9 @@ idg_status launch_degridder_sep(const Geometry &g, const SubgridSet &set, const 
                                 const void *aterms, const float *taper, void *vis_out, void *stream);
 idg_status launch_degridder_sep_fused(const Geometry &g, const SubgridSet &set, const void *grid, const uint8_t *flags,
                                       const void *aterms, const float *taper, void *vis_out, void *stream);
+// the self-test of its failure path: the same launch with MMA threads that give up at once
+idg_status launch_degridder_sep_give_up(const Geometry &g, const SubgridSet &set, const void *grid, const void *aterms,
+                                        const float *taper, void *vis_out, void *stream);
 idg_status read_sepd_error(int *code);
 idg_status launch_gridder_tcw(const Geometry &g, const SubgridSet &set, const void *vis, const uint8_t *flags,
                               const void *aterms, const float *taper, void *subgrids, void *stream);

@@ -14,7 +14,7 @@
 namespace idg {
 namespace tc {
 
-constexpr long kSpin = 1L << 20;                  // polls before a wait gives up (milliseconds at most)
+constexpr long kSpin = 1L << 20;                  // polls before a wait gives up (72 ns each when one thread waits, some us when a CTA does)
 constexpr uint32_t kLBO = 128, kSBO = 256;        // 16 x 16 tile: K-direction and 8-row core-matrix strides
 constexpr int kTile16 = 16 * 32;                  // bytes of a 16-row x 16-K FP16 tile
 
@@ -69,8 +69,8 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(bar) : "memory");
 }
 
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-    for (long it = 0; it < kSpin; ++it) {
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, long polls = kSpin) {
+    for (long it = 0; it < polls; ++it) {
         uint32_t ok;
         asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
                      " selp.u32 %0, 1, 0, p;\n}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
@@ -80,9 +80,10 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
 }
 
 // the same wait without suspending the thread, for the one thread that issues the MMAs (it
-// starts them a little sooner; worker warps that poll cost the others issue slots)
+// starts them a little sooner; worker warps that poll cost the others issue slots).  Its polls are
+// shorter, so there are more
 __device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity) {
-    for (long it = 0; it < kSpin; ++it) {
+    for (long it = 0; it < 16 * kSpin; ++it) {
         uint32_t ok;
         asm volatile("{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
                      " selp.u32 %0, 1, 0, p;\n}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
@@ -90,14 +91,29 @@ __device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity) {
     }
     return false;
 }
-__device__ __forceinline__ void poll_or_fail(uint32_t bar, uint32_t parity, bool &failed) {
-    if (!failed && !mbar_poll(bar, parity)) failed = true;
-}
 
 // a bounded wait that is skipped once this thread has seen a failure, so that
 // control flow stays uniform and the kernel ends
 __device__ __forceinline__ void wait_or_fail(uint32_t bar, uint32_t parity, bool &failed) {
     if (!failed && !mbar_wait(bar, parity)) failed = true;
+}
+
+// The same with a word of the CTA, in shared memory and 0 at the start, that a failure sets: what
+// the CTA writes from then on may rest on data that was not ready.  (A look at the word between the
+// polls, to end all waits with the first, cost the separable kernels 0.5 to 1.3 %; so the limit is
+// lower, about a second when all threads wait.)  NEVER: a self-test's poll that gives up at once.
+__device__ __forceinline__ void wait_or_fail(uint32_t bar, uint32_t parity, bool &failed, volatile int *given_up) {
+    if (!failed && !mbar_wait(bar, parity, kSpin / 4)) {
+        failed = true;
+        *given_up = 1;
+    }
+}
+template <bool NEVER>
+__device__ __forceinline__ void poll_or_fail(uint32_t bar, uint32_t parity, bool &failed, volatile int *given_up) {
+    if (!failed && (NEVER || !mbar_poll(bar, parity))) {
+        failed = true;
+        *given_up = 1;
+    }
 }
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {

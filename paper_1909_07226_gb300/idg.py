@@ -37,7 +37,7 @@ EXPORTED = [
     "idg_autotune", "idg_batch_create", "idg_batch_grid", "idg_batch_degrid", "idg_batch_info",
     "idg_batch_destroy", "idg_device_errors", "idg_taper_window", "idg_taper_aliasing",
     "idg_image_from_grid", "idg_grid_from_image", "idg_plan_set_kernel_variant", "idg_plan_get_kernel_variant",
-    "idg_grid_range", "idg_degrid_range", "idg_selftest_wait_timeout", "idg_aterm_gradient",
+    "idg_grid_range", "idg_degrid_range", "idg_selftest_wait_timeout", "idg_selftest_issue_timeout", "idg_aterm_gradient",
     "idg_classical_grid", "idg_batch_autotune", "idg_grid_degrid_host",
 ]
 BATCH_GRAPH = 1
@@ -122,6 +122,7 @@ def load(path: str = LIB_PATH):
         "idg_batch_destroy": (None, [P]),
         "idg_device_errors": (I32, [P]),
         "idg_selftest_wait_timeout": (I32, [I64, P]),
+        "idg_selftest_issue_timeout": (I32, [P] * 7),
         "idg_taper_window": (I32, [I32, D, I32, P, P]),
         "idg_taper_aliasing": (I32, [I32, D, P, P]),
         "idg_image_from_grid": (I32, [P, P, P, P, P]),
@@ -267,6 +268,18 @@ def device_errors(stream=None):
 def selftest_wait_timeout(max_polls: int = 4096, stream=None):
     """idg_selftest_wait_timeout: enqueue a kernel whose bounded wait runs out on purpose."""
     _check(load().idg_selftest_wait_timeout(int(max_polls), _stream(stream)), "idg_selftest_wait_timeout")
+
+
+def selftest_issue_timeout(plan: Plan, vis, model, aterms, grid_out, vis_out, stream=None):
+    """idg_selftest_issue_timeout: the separable kernels with issuing threads that give up at once."""
+    import torch
+    sh = _shapes(plan)
+    _check(load().idg_selftest_issue_timeout(plan.handle, _dptr(vis, "vis", torch.complex64, sh["vis"]),
+                                             _dptr(model, "model", torch.complex64, sh["grid"]),
+                                             _dptr(aterms, "aterms", torch.complex64, sh["aterms"], True),
+                                             _dptr(grid_out, "grid", torch.complex64, sh["grid"]),
+                                             _dptr(vis_out, "vis_out", torch.complex64, sh["vis"]), _stream(stream)),
+           "idg_selftest_issue_timeout")
 
 
 def autotune(plan, vis, flags, aterms, taper, vis_scratch=None, max_subgrids: int = 4096, stream=None) -> dict:
