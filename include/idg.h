@@ -23,6 +23,9 @@
  *   grid         complex64 [n_w][N][N][4], row index v, column index u;
  *                pixel q of an axis has uv coordinate (q - N/2)/S, S = N * cell;
  *   subgrid      complex64 [L][L][4] (uv or image domain).
+ * Device buffers of complex values start at a multiple of 16 bytes (any allocation does; a slice
+ * may not), visibilities that a call writes as its result (d_vis_out) at one of 8; a buffer that the
+ * kernels chosen for a call cannot address is refused with IDG_ERR_INVALID_ARG.
  * Subgrid image pixel (y, x) sits at l = (x - L/2) S / L, m = (y - L/2) S / L,
  * n' = sqrt(1 - l^2 - m^2) - 1 (Sect. 2, pixel positions; Alg. 1/2 use n').
  *

@@ -360,6 +360,8 @@ struct idg_batch {
     int *d_counters = nullptr;         // one per class
     std::vector<Class> classes;
     std::vector<std::pair<void *, size_t>> zero_on_degrid;   // vis_out of jobs with dropped samples
+    // what check_aligned says of the jobs' buffers for gridding [0] and degridding [1] (empty: aligned)
+    std::string misaligned[2];
     cudaGraphExec_t graph_grid = nullptr, graph_degrid = nullptr;
     cudaStream_t capture_stream = nullptr;   // private stream the graphs are recorded on
 };
@@ -417,6 +419,7 @@ static idg_status batch_run(idg_batch *b, bool degrid, idg_stream stream) {
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
     if (dev != b->device) return fail(IDG_ERR_INVALID_ARG, "the batch belongs to another device");
+    if (!b->misaligned[degrid].empty()) return fail(IDG_ERR_INVALID_ARG, b->misaligned[degrid]);
     cudaStream_t s = (cudaStream_t)stream;
     if (!(b->flags & IDG_BATCH_GRAPH)) return batch_enqueue(b, degrid, s);
     cudaGraphExec_t &exec = degrid ? b->graph_degrid : b->graph_grid;
@@ -522,6 +525,17 @@ idg_status idg_batch_create(const idg_plan *const *plans, const idg_job_buffers 
         J.aterms = (const float4 *)bufs[j].aterms;
         J.taper = p->taper_or_default(bufs[j].taper);
         J.grid = (float4 *)bufs[j].grid;
+        // (the separable kernels add 8 bytes at a time to the grid, the others 16)
+        bool all_sep = separable_size(p->L);
+        for (int64_t s = 0; s < p->stats.n_subgrids; ++s) all_sep = all_sep && (p->split_sub[s] || p->sep_sub[s]);
+        if (p->stats.n_subgrids > 0)
+            for (int dir = 0; dir < 2; ++dir) {
+                const Buffer vis{dir ? bufs[j].vis_out : bufs[j].vis, dir ? "vis_out" : "vis", dir ? 8u : 16u};
+                const Buffer grid{bufs[j].grid, "grid", !dir && all_sep ? 8u : 16u};
+                if (b->misaligned[dir].empty() &&
+                    check_aligned({vis, {bufs[j].aterms, "aterms", 16}, grid}) != IDG_OK)
+                    b->misaligned[dir] = "job " + std::to_string(j) + ": " + idg_last_error();
+            }
         b->n_vis += p->stats.n_vis_planned;
         if (p->any_dropped && bufs[j].vis_out)
             b->zero_on_degrid.push_back({bufs[j].vis_out, (size_t)p->n_bl * p->n_t * p->n_chan * 32});
@@ -669,6 +683,10 @@ idg_status idg_batch_autotune(idg_batch *b, double *ms, int cap, idg_stream stre
             KernelShape &cur = dir ? cl.degrid : cl.grid;
             int &cur_blocks = dir ? cl.degrid_blocks : cl.grid_blocks;
             if (cl.n_items == 0 || cur.tc) continue;     // the tensor-core classes have one shape
+            if (!b->misaligned[dir].empty()) {
+                st = fail(IDG_ERR_INVALID_ARG, b->misaligned[dir]);
+                break;
+            }
             const auto shapes = dir ? degrid_shapes(cl.L) : grid_shapes(cl.L);
             double best_ms = 1e300;
             for (const KernelShape &x : shapes) {

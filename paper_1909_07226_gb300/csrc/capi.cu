@@ -31,6 +31,14 @@ idg_status cuda_fail(int err, const char *what) {
     return err == cudaErrorMemoryAllocation ? IDG_ERR_NO_MEMORY : IDG_ERR_CUDA;
 }
 
+idg_status check_aligned(std::initializer_list<Buffer> buffers) {
+    for (const Buffer &b : buffers)
+        if ((uintptr_t)b.ptr % b.bytes)
+            return fail(IDG_ERR_INVALID_ARG,
+                        std::string(b.name) + " must start at a multiple of " + std::to_string(b.bytes) + " bytes");
+    return IDG_OK;
+}
+
 idg_status launch_subgrid_fft(const idg_plan *p, int64_t count, int direction, void *subgrids, void *stream) {
     if (p->opts.fft_mode == IDG_FFT_TC_SPLIT) return launch_dft_tc(p->L, count, direction, subgrids, stream);
     return launch_fft(p->L, count, direction, subgrids, stream);
@@ -905,10 +913,16 @@ static idg_status no_default_taper() {
     return fail(IDG_ERR_INVALID_ARG, "the taper is NULL and the plan has no default taper");
 }
 
-static idg_status check_call(const idg_plan *p, const void *a, const char *an, const void *b, const char *bn) {
+// (buffers: checked where a kernel will touch them, over `count` subgrids, -1: the plan's)
+static idg_status check_call(const idg_plan *p, const void *a, const char *an, const void *b, const char *bn,
+                             std::initializer_list<Buffer> buffers = {}, int64_t count = -1) {
     if (!p) return fail(IDG_ERR_INVALID_ARG, "plan is NULL");
     if (!a) return fail(IDG_ERR_INVALID_ARG, std::string(an) + " is NULL");
     if (!b) return fail(IDG_ERR_INVALID_ARG, std::string(bn) + " is NULL");
+    if ((count < 0 ? p->stats.n_subgrids : count) > 0) {
+        const idg_status st = check_aligned(buffers);
+        if (st != IDG_OK) return st;
+    }
     if (!gridder_supported(p->L))
         return fail(IDG_ERR_UNSUPPORTED, "subgrid size " + std::to_string(p->L) + " is not compiled in");
     return check_device(p);
@@ -1059,6 +1073,13 @@ static bool spans_need_scratch(const idg_plan *p, bool grid) {
     return false;
 }
 
+// the alignment of a gridding call's grid: the fused separable kernel adds 8 bytes at a time, every
+// other adder 16
+static Buffer grid_out(const idg_plan *p, Order o, int64_t first, int64_t count, const void *grid) {
+    const bool eight = count == 0 || (sep_head(p, o, first, count) == count && fused_grid(p, true));
+    return Buffer{grid, "d_grid", eight ? 8u : 16u};
+}
+
 // Grid the subgrids at positions [first, first + count) of the order o, all of one
 // kind (g.separable), in pieces of at most `chunk` subgrids that pass through the
 // subgrid scratch (gridder -> transform -> adder), or in one fused launch (no scratch).
@@ -1169,7 +1190,8 @@ static idg_status grid_call(const idg_plan *p, Order o, int64_t first, int64_t c
                             const uint8_t *flags, const void *aterms, const float *taper, void *grid,
                             cudaStream_t s) {
     if (count == 0) return IDG_OK;
-    idg_status st = IDG_OK;
+    idg_status st = check_aligned({grid_out(p, o, first, count, grid)});
+    if (st != IDG_OK) return st;
     const int64_t chunk = std::min(chunk_subgrids(p), count);
     const bool comp = p->opts.adder_mode == IDG_ADDER_COMPENSATED;
     void *scratch = nullptr;     // the subgrid scratch, unless fused launches take the call
@@ -1216,7 +1238,9 @@ static idg_status degrid_call(const idg_plan *p, Order o, int64_t first, int64_t
 idg_status idg_aterm_gradient(const idg_plan *p, const void *grid, const void *vis, const uint8_t *flags,
                               const void *aterms, const float *taper, void *residual, void *gradient, double *cost,
                               idg_stream stream) {
-    idg_status st = check_call(p, grid, "d_grid", vis, "d_vis");
+    idg_status st = check_call(p, grid, "d_grid", vis, "d_vis",
+                               {{grid, "d_grid", 16}, {vis, "d_vis", 16}, {aterms, "d_aterms", 16},
+                                {residual, "d_residual", 16}, {gradient, "d_gradient", 16}});
     if (st != IDG_OK) return st;
     if (!residual) return fail(IDG_ERR_INVALID_ARG, "d_residual is NULL");
     if (!gradient) return fail(IDG_ERR_INVALID_ARG, "d_gradient is NULL");
@@ -1272,7 +1296,7 @@ idg_status idg_aterm_gradient(const idg_plan *p, const void *grid, const void *v
 
 idg_status idg_grid(const idg_plan *p, const void *vis, const uint8_t *flags, const void *aterms,
                     const float *taper, void *grid, idg_stream stream) {
-    idg_status st = check_call(p, vis, "d_vis", grid, "d_grid");
+    idg_status st = check_call(p, vis, "d_vis", grid, "d_grid", {{vis, "d_vis", 16}, {aterms, "d_aterms", 16}});
     if (st != IDG_OK) return st;
     if (!(taper = p->taper_or_default(taper))) return no_default_taper();
     const Lists ls = lists_for(p, true);
@@ -1281,7 +1305,8 @@ idg_status idg_grid(const idg_plan *p, const void *vis, const uint8_t *flags, co
 
 idg_status idg_degrid(const idg_plan *p, const void *grid, const uint8_t *flags, const void *aterms,
                       const float *taper, void *vis_out, idg_stream stream) {
-    idg_status st = check_call(p, grid, "d_grid", vis_out, "d_vis_out");
+    idg_status st = check_call(p, grid, "d_grid", vis_out, "d_vis_out",
+                               {{grid, "d_grid", 16}, {aterms, "d_aterms", 16}, {vis_out, "d_vis_out", 8}});
     if (st != IDG_OK) return st;
     if (!(taper = p->taper_or_default(taper))) return no_default_taper();
     cudaStream_t s = (cudaStream_t)stream;
@@ -1296,7 +1321,7 @@ idg_status idg_degrid(const idg_plan *p, const void *grid, const uint8_t *flags,
 
 idg_status idg_grid_range(const idg_plan *p, int64_t first, int64_t count, const void *vis, const uint8_t *flags,
                           const void *aterms, const float *taper, void *grid, idg_stream stream) {
-    idg_status st = check_call(p, vis, "d_vis", grid, "d_grid");
+    idg_status st = check_call(p, vis, "d_vis", grid, "d_grid", {{vis, "d_vis", 16}, {aterms, "d_aterms", 16}}, count);
     if (st != IDG_OK) return st;
     if (!(taper = p->taper_or_default(taper))) return no_default_taper();
     if ((st = check_range(p, first, count)) != IDG_OK) return st;
@@ -1305,7 +1330,8 @@ idg_status idg_grid_range(const idg_plan *p, int64_t first, int64_t count, const
 
 idg_status idg_degrid_range(const idg_plan *p, int64_t first, int64_t count, const void *grid, const uint8_t *flags,
                             const void *aterms, const float *taper, void *vis_out, idg_stream stream) {
-    idg_status st = check_call(p, grid, "d_grid", vis_out, "d_vis_out");
+    idg_status st = check_call(p, grid, "d_grid", vis_out, "d_vis_out",
+                               {{grid, "d_grid", 16}, {aterms, "d_aterms", 16}, {vis_out, "d_vis_out", 8}}, count);
     if (st != IDG_OK) return st;
     if (!(taper = p->taper_or_default(taper))) return no_default_taper();
     if ((st = check_range(p, first, count)) != IDG_OK) return st;
@@ -1628,7 +1654,9 @@ idg_status idg_grid_degrid_host(const idg_plan *p, const void *h_vis, const void
 
 idg_status idg_selftest_issue_timeout(const idg_plan *p, const void *vis, const void *model, const void *aterms,
                                       void *grid, void *vis_out, idg_stream stream) {
-    idg_status st = check_call(p, vis, "d_vis", grid, "d_grid");
+    idg_status st = check_call(p, vis, "d_vis", grid, "d_grid",
+                               {{vis, "d_vis", 16}, {model, "d_model", 16}, {aterms, "d_aterms", 16},
+                                {grid, "d_grid", 8}, {vis_out, "d_vis_out", 8}});
     if (st != IDG_OK) return st;
     if (!model) return fail(IDG_ERR_INVALID_ARG, "d_model is NULL");
     if (!vis_out) return fail(IDG_ERR_INVALID_ARG, "d_vis_out is NULL");
@@ -1649,7 +1677,8 @@ idg_status idg_selftest_issue_timeout(const idg_plan *p, const void *vis, const 
 idg_status idg_grid_subgrids(const idg_plan *p, int64_t first, int64_t count, const void *vis,
                              const uint8_t *flags, const void *aterms, const float *taper, void *sub,
                              idg_stream stream) {
-    idg_status st = check_call(p, vis, "d_vis", sub, "d_subgrids");
+    idg_status st = check_call(p, vis, "d_vis", sub, "d_subgrids",
+                               {{vis, "d_vis", 16}, {aterms, "d_aterms", 16}, {sub, "d_subgrids", 16}}, count);
     if (st != IDG_OK) return st;
     if (!(taper = p->taper_or_default(taper))) return no_default_taper();
     if ((st = check_range(p, first, count)) != IDG_OK || count == 0) return st;
@@ -1659,7 +1688,7 @@ idg_status idg_grid_subgrids(const idg_plan *p, int64_t first, int64_t count, co
 }
 
 idg_status idg_fft_subgrids(const idg_plan *p, int64_t count, int direction, void *sub, idg_stream stream) {
-    idg_status st = check_call(p, sub, "d_subgrids", sub, "d_subgrids");
+    idg_status st = check_call(p, sub, "d_subgrids", sub, "d_subgrids", {{sub, "d_subgrids", 16}}, count);
     if (st != IDG_OK) return st;
     if (direction != -1 && direction != 1) return fail(IDG_ERR_INVALID_ARG, "direction must be -1 or +1");
     if (count < 0) return fail(IDG_ERR_INVALID_ARG, "count < 0");
@@ -1670,7 +1699,8 @@ idg_status idg_fft_subgrids(const idg_plan *p, int64_t count, int direction, voi
 
 idg_status idg_add_subgrids(const idg_plan *p, int64_t first, int64_t count, const void *sub, void *grid,
                             idg_stream stream) {
-    idg_status st = check_call(p, sub, "d_subgrids", grid, "d_grid");
+    idg_status st = check_call(p, sub, "d_subgrids", grid, "d_grid",
+                               {{sub, "d_subgrids", 16}, {grid, "d_grid", 16}}, count);
     if (st != IDG_OK) return st;
     if ((st = check_range(p, first, count)) != IDG_OK || count == 0) return st;
     ProfileScope ps(IDG_KERNEL_ADDER, stream, 96.0 * pixels(p, count));
@@ -1681,7 +1711,8 @@ idg_status idg_add_subgrids(const idg_plan *p, int64_t first, int64_t count, con
 
 idg_status idg_split_subgrids(const idg_plan *p, int64_t first, int64_t count, const void *grid, void *sub,
                               idg_stream stream) {
-    idg_status st = check_call(p, grid, "d_grid", sub, "d_subgrids");
+    idg_status st = check_call(p, grid, "d_grid", sub, "d_subgrids",
+                               {{grid, "d_grid", 16}, {sub, "d_subgrids", 16}}, count);
     if (st != IDG_OK) return st;
     if ((st = check_range(p, first, count)) != IDG_OK || count == 0) return st;
     ProfileScope ps(IDG_KERNEL_SPLITTER, stream, 64.0 * pixels(p, count));
@@ -1691,7 +1722,8 @@ idg_status idg_split_subgrids(const idg_plan *p, int64_t first, int64_t count, c
 idg_status idg_degrid_subgrids(const idg_plan *p, int64_t first, int64_t count, const void *sub,
                                const uint8_t *flags, const void *aterms, const float *taper, void *vis_out,
                                idg_stream stream) {
-    idg_status st = check_call(p, sub, "d_subgrids", vis_out, "d_vis_out");
+    idg_status st = check_call(p, sub, "d_subgrids", vis_out, "d_vis_out",
+                               {{sub, "d_subgrids", 16}, {aterms, "d_aterms", 16}, {vis_out, "d_vis_out", 8}}, count);
     if (st != IDG_OK) return st;
     if (!(taper = p->taper_or_default(taper))) return no_default_taper();
     if ((st = check_range(p, first, count)) != IDG_OK || count == 0) return st;
@@ -1768,7 +1800,8 @@ int idg_plan_get_kernel_variant(const idg_plan *p, int kernel) {
 idg_status idg_autotune(const idg_plan *p, const void *vis, const uint8_t *flags, const void *aterms,
                         const float *taper, void *vis_scratch, int64_t max_subgrids, double *gridder_ms,
                         double *degridder_ms, int cap, idg_stream stream) {
-    idg_status st = check_call(p, vis, "d_vis", vis, "d_vis");
+    idg_status st = check_call(p, vis, "d_vis", vis, "d_vis",
+                               {{vis, "d_vis", 16}, {aterms, "d_aterms", 16}, {vis_scratch, "d_vis_scratch", 8}});
     if (st != IDG_OK) return st;
     if (!(taper = p->taper_or_default(taper))) return no_default_taper();
     const int64_t n = p->stats.n_subgrids;

@@ -411,6 +411,10 @@ extern "C" idg_status idg_classical_grid(const idg_plan *p, int M, int O, double
         return fail(IDG_ERR_INVALID_ARG, "oversample^2 * support^2 * 128 bytes (one kernel) exceeds 256 MiB");
     if (classical_grid_smem(p->L, M) > 200 * 1024)
         return fail(IDG_ERR_UNSUPPORTED, "subgrid size + support too large for the shared-memory tile");
+    if (p->stats.n_subgrids > 0) {
+        const idg_status st = check_aligned({{vis, "d_vis", 16}, {aterms, "d_aterms", 8}, {grid, "d_grid", 16}});
+        if (st != IDG_OK) return st;
+    }
     if (p->device < 0) return fail(IDG_ERR_INVALID_ARG, "the plan was created without a CUDA device");
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);

@@ -103,8 +103,7 @@ __device__ __forceinline__ void degrid_write(const Geometry &g, const DevSubgrid
                 o01 = make_float4(0.f, 0.f, 0.f, 0.f);
                 o23 = o01;
             }
-            vis_out[2 * vi] = o01;
-            vis_out[2 * vi + 1] = o23;
+            store_vis(vis_out, vi, o01, o23);
         }
     }
 }

@@ -411,8 +411,8 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
                 float4 v = make_float4((own.x + o.x) * inv_scale, (own.y + o.y) * inv_scale, (own.z + o.z) * inv_scale,
                                        (own.w + o.w) * inv_scale);
                 if (ovi & 0x80000000u) v = make_float4(0.f, 0.f, 0.f, 0.f);      // flagged
-                // as two 8-byte stores: a complex64 output may start at any multiple of 8 bytes (one
-                // 16-byte store took the same time)
+                // as two 8-byte stores: a complex64 output may start at any multiple of 8 bytes (the other
+                // degridders choose by the address, store_vis; here one 16-byte store took the same time)
                 float2 *out = (float2 *)vis_out + 4 * (size_t)(ovi & 0x7FFFFFFFu) + 2 * half;
                 out[0] = make_float2(v.x, v.y);
                 out[1] = make_float2(v.z, v.w);

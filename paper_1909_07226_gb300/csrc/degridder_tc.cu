@@ -251,8 +251,7 @@ __device__ __forceinline__ void degridder_tcw_body(const Geometry &g, const DevS
                     o01 = make_float4(0.f, 0.f, 0.f, 0.f);
                     o23 = o01;
                 }
-                vis_out[2 * vi] = o01;
-                vis_out[2 * vi + 1] = o23;
+                store_vis(vis_out, vi, o01, o23);
             }
 #pragma unroll
             for (int c = 0; c < 8; ++c) acc[c] = 0.0f;

@@ -75,7 +75,22 @@ __device__ __forceinline__ void red_add_f4(float4 *p, float4 v) {
                  : "memory");
 }
 
-// the same for 8 bytes
+// a visibility's four polarisations a, b.  A complex64 array may start at any multiple of 8 bytes, and
+// 16-byte stores need one of 16: the branch is the same for every thread
+__device__ __forceinline__ void store_vis(float4 *out, size_t vi, float4 a, float4 b) {
+    if (((size_t)out & 15) == 0) {
+        out[2 * vi] = a;
+        out[2 * vi + 1] = b;
+    } else {
+        float2 *o = (float2 *)out + 4 * vi;
+        o[0] = make_float2(a.x, a.y);
+        o[1] = make_float2(a.z, a.w);
+        o[2] = make_float2(b.x, b.y);
+        o[3] = make_float2(b.z, b.w);
+    }
+}
+
+// *p += v as one 8-byte reduction
 __device__ __forceinline__ void red_add_f2(float2 *p, float2 v) {
     asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" :: "l"(p), "f"(v.x), "f"(v.y) : "memory");
 }

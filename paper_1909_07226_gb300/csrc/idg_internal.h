@@ -3,6 +3,7 @@
 
 #include <atomic>
 #include <cstdint>
+#include <initializer_list>
 #include <string>
 #include <vector>
 
@@ -184,6 +185,15 @@ idg_status scratch_alloc(int device, size_t bytes, void *stream, void **p);
 void set_error(const std::string &msg);
 idg_status fail(idg_status st, const std::string &msg);
 idg_status cuda_fail(int err, const char *what);
+
+// a caller's device buffer that kernels read or write `bytes` bytes at a time (ptr NULL: not used);
+// a misaligned one would be an addressing error on the device, so it is refused here
+struct Buffer {
+    const void *ptr;
+    const char *name;
+    unsigned bytes;
+};
+idg_status check_aligned(std::initializer_list<Buffer> buffers);
 
 // event-based kernel timing (idg_profile_*); no-ops while disabled
 struct ProfileScope {

@@ -766,6 +766,13 @@ idg_status image_setup(const idg_plan *p, const void *a_ptr, const void *b_ptr, 
     if (!p || !a_ptr || !b_ptr) return fail(IDG_ERR_INVALID_ARG, "plan, input and output are required");
     const int N = p->N;
     if (N < 32 || N > 4096 || (N & (N - 1))) return fail(IDG_ERR_UNSUPPORTED, "the image transform needs N a power of two, 32 .. 4096");
+    // every pass moves 16 bytes at a time, at N = 4096 all but the read of the image 8
+    if (p->stats.n_w_layers > 0) {
+        const unsigned in = N == 4096 && sign > 0 ? 8 : 16, out = N == 4096 ? 8 : 16;
+        const idg_status st = check_aligned({{a_ptr, sign > 0 ? "d_grid" : "d_image", in},
+                                             {b_ptr, sign > 0 ? "d_image" : "d_grid", out}});
+        if (st != IDG_OK) return st;
+    }
     logN = 0;
     while ((1 << logN) < N) ++logN;
     int dev = -1;

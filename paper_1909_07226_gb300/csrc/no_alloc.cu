@@ -72,6 +72,10 @@ extern "C" idg_status idg_grid_no_alloc(const idg_plan *p, const void *vis, cons
         return fail(IDG_ERR_UNSUPPORTED,
                     "idg_grid_no_alloc: the compensated adder needs a grid-sized buffer that this call cannot "
                     "allocate; use a plan with IDG_ADDER_ATOMIC or idg_grid");
+    if (p->stats.n_subgrids > 0) {
+        const idg_status st = check_aligned({{vis, "d_vis", 16}, {aterms, "d_aterms", 16}, {grid, "d_grid", 16}});
+        if (st != IDG_OK) return st;
+    }
     if (!gridder_supported(p->L))
         return fail(IDG_ERR_UNSUPPORTED, "subgrid size " + std::to_string(p->L) + " is not compiled in");
     if (p->device < 0) return fail(IDG_ERR_INVALID_ARG, "the plan was created without a CUDA device");

@@ -256,8 +256,7 @@ degridder_rec_kernel(Geometry g, const int32_t *__restrict__ idx, int64_t first,
                         o01 = make_float4(0.f, 0.f, 0.f, 0.f);
                         o23 = o01;
                     }
-                    vis_out[2 * vi] = o01;
-                    vis_out[2 * vi + 1] = o23;
+                    store_vis(vis_out, vi, o01, o23);
                 }
             }
         }
