@@ -46,9 +46,9 @@ ISSUE_PER_VISPIX_TC = 9
 # DRAM bytes (read + write) per visibility-pixel of one launch, from the ncu
 # capture of the separable kernels (the default at L = 32 where the plan is
 # separable) on the LOFAR-like slice, one launch of all its subgrids, 4.731e9
-# visibility-pixels: gridder 178.5 MB (visibilities and coordinates in; the
+# visibility-pixels: gridder 178.2 MB (visibilities and coordinates in; the
 # atomically updated grid lines are still dirty in L2 when the launch ends), degridder
-# 120.8 MB
+# 120.4 MB
 # (grid lines and coordinates in, model visibilities out).  The traffic is
 # proportional to the work, so it scales to a full launch by the units processed.
 # Kernels without a capture of their current code report no traffic.
@@ -56,8 +56,9 @@ FUSED_VARIANT = "tcgen05_tmemA_ws_nt288_fused"
 SEP_VARIANT = "tcgen05_separable_fused"
 # Tensor-core work of the separable kernels at subgrid size L (kind::f16, M = 128, K = 16
 # per MMA, 2 FLOP per multiply-add): the gridder issues N = 6 L + 2 L per group of 8
-# visibilities (192 + 64 at L = 32), the degridder L / 8 K steps of 4 x N = 4 L per tile
-# of 64 visibilities.
+# visibilities (192 + 64 at L = 32), the degridder L / 8 K steps of 4 x N = 8 L per tile of
+# 128 visibilities (at L = 32 and 24 in two rounds of two polarisations).
+SEP_DEGRID_TILE = 128
 
 
 def sep_grid_flop_per_group(L):
@@ -65,11 +66,11 @@ def sep_grid_flop_per_group(L):
 
 
 def sep_degrid_flop_per_tile(L):
-    return (L // 8) * 4 * 2 * 128 * 16 * (4 * L)
+    return (L // 8) * 4 * 2 * 128 * 16 * (8 * L)
 
 # Half of those products are the FP16 hi/lo split that keeps FP32 accuracy: the
 # gridder's N = 256 columns are A_hi x [B_hi (128) | B0_lo (64)] and A_lo x B0_hi (64);
-# the degridder's four N = 128 products per K step are hi x hi of the m = 0 and the
+# the degridder's four products per K step are hi x hi of the m = 0 and the
 # first-order w term plus the two lo corrections of the m = 0 term.  The method's own
 # contraction (hi x hi) is the other half.
 SEP_USEFUL_SHARE = 0.5
@@ -77,8 +78,8 @@ DTYPE_SEP = "f32 (fp16 hi/lo split tensor-core products, fp32 accumulate)"
 DTYPE_MIXED = ("f32 (fp16 hi/lo split tensor-core products for subgrids within the separable bound and "
                "pieces, packed fp32 for the rest; fp32 accumulate)")
 KERNEL_TRAFFIC = {
-    "gridder": {SEP_VARIANT: 178.5e6 / 4.731e9},
-    "degridder": {SEP_VARIANT: 120.8e6 / 4.731e9},
+    "gridder": {SEP_VARIANT: 178.2e6 / 4.731e9},
+    "degridder": {SEP_VARIANT: 120.4e6 / 4.731e9},
 }
 
 
@@ -501,7 +502,7 @@ def run_gb300(args, world, rank, local):
     bf16_src = "measured burst" if "bf16_tflops" in peaks else "fallback"
     kp = plan.export()[:, 9].astype(np.int64)                 # K_p per subgrid (descriptor field 9)
     sep_flop = {"gridder": float(((kp + 7) // 8).sum()) * sep_grid_flop_per_group(wl.subgrid_size),
-                "degridder": float(((kp + 63) // 64).sum()) * sep_degrid_flop_per_tile(wl.subgrid_size)}
+                "degridder": float((-(-kp // SEP_DEGRID_TILE)).sum()) * sep_degrid_flop_per_tile(wl.subgrid_size)}
     kernels = {}
     for k, d in prof.items():
         if d["launches"] == 0:
@@ -551,7 +552,7 @@ def run_gb300(args, world, rank, local):
     if "achieved_vispix" in kernels[dom]:
         roof["achieved_vispix"] = kernels[dom]["achieved_vispix"]
         roof["flop_basis"] = ("MMA FLOP issued: gridder 2*128*16*8L per group of 8 visibilities, degridder "
-                              "(L/8)*4*2*128*16*4L per tile of 64 (FP16 hi/lo split products included)")
+                              "(L/8)*4*2*128*16*8L per tile of 128 (FP16 hi/lo split products included)")
     gpu_launches = int(sum(d["launches"] for d in prof.values()))
 
     # image-side steps, outside the grid + degrid step: the whole grid to the image and
