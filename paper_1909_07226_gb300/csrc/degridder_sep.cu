@@ -45,8 +45,9 @@
 //   this layout                                               8.35       4.69
 //   constants instead of tables                               8.04       4.53
 //   one thread per transform line, straight from the rows     7.92       4.36
-//   A-terms two pixels ahead                                  7.93       4.15
-// The tensor pipe is 50 % busy (16 cycles per visibility at full rate), issue slots 46 %: a
+//   A-terms two pixels ahead                                  7.93       4.24
+//   failures seen by every store                              7.88       4.27
+// The tensor pipe is 49 % busy (16 cycles per visibility at full rate), issue slots 46 %: a
 // CTA's chain per tile (A 1250, MMAs 2 x 1024, sums 2 x 500 cycles, measured alone) leaves
 // the tensor cores to the other CTA for just over half its length, and tensor memory has no
 // room for a second A beside the accumulator.  Short subgrids are bound by the prologue
@@ -134,27 +135,27 @@ __device__ __forceinline__ void form_a(const Geometry &g, uint32_t lane_base, fl
     const float cz = cc * csig;
     const f2_t cz2 = f2_pack(cz, cz), nz2 = f2_pack(-cz, -cz);
 #pragma unroll
-        for (int x0 = X0; x0 < X0 + H; x0 += XCH) {
-            uint32_t hi[XCH], lo[XCH], m1[XCH];
+    for (int x0 = X0; x0 < X0 + H; x0 += XCH) {
+        uint32_t hi[XCH], lo[XCH], m1[XCH];
 #pragma unroll
-            for (int i = 0; i < XCH; i += 2) {
-                float sn0, cs0, sn1, cs1;
-                __sincosf(fmaf(cc, g.sep_s[x0 + i], ca * (float)(x0 + i - SL / 2)), &sn0, &cs0);
-                __sincosf(fmaf(cc, g.sep_s[x0 + i + 1], ca * (float)(x0 + i + 1 - SL / 2)), &sn1, &cs1);
-                const f2_t c2 = f2_pack(cs0, cs1), s2 = f2_pack(sn0, sn1);
-                f2_t hc, lc, hs, ls;
-                f2_split(c2, magic_1, hc, lc);
-                f2_split(s2, magic_1, hs, ls);
-                pack_pairs(hc, hs, hi[i], hi[i + 1]);
-                pack_pairs(lc, ls, lo[i], lo[i + 1]);
-                pack_pairs(f2_mul(nz2, s2), f2_mul(cz2, c2), m1[i], m1[i + 1]);
-            }
-            const uint32_t ta = lane_base + C::A_COL + (uint32_t)x0;
-            tmem_st(ta, hi);
-            tmem_st(ta + SL, lo);
-            tmem_st(ta + 2 * SL, m1);
+        for (int i = 0; i < XCH; i += 2) {
+            float sn0, cs0, sn1, cs1;
+            __sincosf(fmaf(cc, g.sep_s[x0 + i], ca * (float)(x0 + i - SL / 2)), &sn0, &cs0);
+            __sincosf(fmaf(cc, g.sep_s[x0 + i + 1], ca * (float)(x0 + i + 1 - SL / 2)), &sn1, &cs1);
+            const f2_t c2 = f2_pack(cs0, cs1), s2 = f2_pack(sn0, sn1);
+            f2_t hc, lc, hs, ls;
+            f2_split(c2, magic_1, hc, lc);
+            f2_split(s2, magic_1, hs, ls);
+            pack_pairs(hc, hs, hi[i], hi[i + 1]);
+            pack_pairs(lc, ls, lo[i], lo[i + 1]);
+            pack_pairs(f2_mul(nz2, s2), f2_mul(cz2, c2), m1[i], m1[i + 1]);
         }
-        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        const uint32_t ta = lane_base + C::A_COL + (uint32_t)x0;
+        tmem_st(ta, hi);
+        tmem_st(ta + SL, lo);
+        tmem_st(ta + 2 * SL, m1);
+    }
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
 // Ey* of its y from Y0 as pairs (cs_y, cs_y+1), (sn_y, sn_y+1)
@@ -162,13 +163,13 @@ template <int L, int Y0>
 __device__ __forceinline__ void form_ey(const Geometry &g, float cb, float cc, f2_t (&ec)[L / 4], f2_t (&es)[L / 4]) {
     constexpr int SL = L, H = L / 2;
 #pragma unroll
-        for (int j = 0; j < H / 2; ++j) {
-            float s0, c0, s1, c1;
-            __sincosf(fmaf(cc, g.sep_t[Y0 + 2 * j], cb * (float)(Y0 + 2 * j - SL / 2)), &s0, &c0);
-            __sincosf(fmaf(cc, g.sep_t[Y0 + 2 * j + 1], cb * (float)(Y0 + 2 * j + 1 - SL / 2)), &s1, &c1);
-            ec[j] = f2_pack(c0, c1);
-            es[j] = f2_pack(s0, s1);
-        }
+    for (int j = 0; j < H / 2; ++j) {
+        float s0, c0, s1, c1;
+        __sincosf(fmaf(cc, g.sep_t[Y0 + 2 * j], cb * (float)(Y0 + 2 * j - SL / 2)), &s0, &c0);
+        __sincosf(fmaf(cc, g.sep_t[Y0 + 2 * j + 1], cb * (float)(Y0 + 2 * j + 1 - SL / 2)), &s1, &c1);
+        ec[j] = f2_pack(c0, c1);
+        es[j] = f2_pack(s0, s1);
+    }
 }
 
 // Visibilities of subgrid d of geometry g from its image src[L][L][4], or with
@@ -405,9 +406,9 @@ __device__ __forceinline__ void degridder_sep_body(const Geometry &g, const DevS
         uint32_t ovi = 0xFFFFFFFFu;
         auto finish = [&](int t) {
             pair_sync(quarter);
-            const bool lost = *(const volatile int *)&s_given_up;     // (also what the other half saw before)
             const float4 o = s_part[((t & 1) * 2 + half) * TV + row];
-            if (ovi != 0xFFFFFFFFu && !lost) {
+            // (read after the pair has met: a wait of the other half that ran out counts too)
+            if (ovi != 0xFFFFFFFFu && !s_given_up) {
                 float4 v = make_float4((own.x + o.x) * inv_scale, (own.y + o.y) * inv_scale, (own.z + o.z) * inv_scale,
                                        (own.w + o.w) * inv_scale);
                 if (ovi & 0x80000000u) v = make_float4(0.f, 0.f, 0.f, 0.f);      // flagged

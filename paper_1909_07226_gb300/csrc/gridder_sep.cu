@@ -73,9 +73,10 @@
 //   two rows x two polarisations per thread                  11.28       4.73
 //   A's hi by its own size, rounded per polarisation (the
 //   figures above: one quantum per subgrid)                  11.41       4.84
-// It is bound by latency and issue of the producers together: issue slots 56 %, the
-// shared-memory data pipe 52 %, the tensor pipe 35 % busy; leaving out any one of the
-// V loads, the split, the phasors or the MMA width gains 1 to 10 %.  Measured and not
+//   the waits' failure word (the code it generates)          11.15       4.78
+// It is bound by latency and issue of the producers together (busy: issue slots 62 %, the
+// shared-memory data pipe 52 %, the tensor pipe 35 %); leaving out any one of the
+// V loads, the split, the phasors or the MMA width gained 1 to 10 %.  Measured and not
 // kept: A's hi rounded in FP32 with float means (11.72 and 4.94 ms: more registers, and the sums'
 // shuffles weigh on short subgrids); one group per stage with two buffers (a stage's hand-over costs each warp
 // about 670 cycles: 15.7 ms), polling by the producers (13.2), eight columns per fold
@@ -619,7 +620,7 @@ __device__ __forceinline__ void gridder_sep_body(const Geometry &g, const DevSub
     const bool lost = __syncthreads_or(failed);
     if (lost && tid == 0) atomicExch(&g_sep_error, 1);
     if (!lost) {
-        // image-domain kernel per pixel: taper * A_p^H I A_q (with the centring factor when FUSED)
+        // image-domain kernel per pixel: taper * A_p^H I A_q (the transform's lines centre themselves)
         if (producer) {
 #pragma unroll
             for (int ip = 0; ip < PIXT; ++ip) {
