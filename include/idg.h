@@ -580,7 +580,8 @@ idg_status idg_autotune(const idg_plan *plan, const void *d_vis, const uint8_t *
  * wait on shared-memory barriers for their matrix operations and bulk copies;
  * every wait has an iteration limit, after which the kernel records an error
  * in a device word, waits (bounded) for its own operations in flight, releases
- * its tensor memory and leaves its outputs unwritten.  idg_device_errors
+ * its tensor memory and writes nothing more (a degridder may have written the
+ * subgrid's first visibilities before the wait).  idg_device_errors
  * synchronises `stream`, reads and clears the words, and returns
  * IDG_ERR_TIMEOUT if any wait gave up since the last call, else
  * IDG_ERR_DEVICE_CHECK if a device-side check failed (the classical gridder
